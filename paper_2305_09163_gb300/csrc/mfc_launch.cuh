@@ -9,9 +9,26 @@ namespace mfc {
 constexpr int kSweepThreads = 128;
 constexpr int kElemThreads = 256;
 
-// Slots (edge cells) owned by one CTA of the x-stream kernel: 16 chunks of 128,
-// so the two recomputed slots at its start cost about 0.1%.
-constexpr long long kStreamSlotsPerBlock = 16LL * kStreamThreads;
+// Chunks of kStreamThreads slots (edge cells) that one CTA of the x-stream
+// kernel walks.  A CTA starts two slots early (both faces of its first cell), so
+// k chunks finish 128 k - 2 slots; owning exactly that many leaves no nearly
+// empty last chunk (2,048 owned slots took 17 chunks for the work of 16.02).
+// Long runs save those two slots, short ones fill the chip: a chunk takes ~10 us
+// alone on an SM and ~4.3 us with four CTAs sharing it, and with the fixed 16
+// chunks a 1000-cell row ran on one SM (79 us per launch) and a 65,000-cell block
+// on half of them.  So k grows only once every SM has 16 CTAs to run, four
+// times what it holds, where the walk's end is a small part; past 16 the two
+// slots are 0.1% and nothing is left to save.
+constexpr long long kStreamMaxChunks = 16;
+constexpr long long kStreamMinBlocks = 152LL * 16;
+
+inline long long stream_slots_per_block(long long total) {
+    const long long chunks = (total + kStreamThreads - 3) / (kStreamThreads - 2);
+    long long k = chunks / kStreamMinBlocks;
+    if (k < 1) k = 1;
+    if (k > kStreamMaxChunks) k = kStreamMaxChunks;
+    return k * kStreamThreads - 2;
+}
 
 inline size_t stage_bytes_rt(int mask, int nq, size_t real_size) {
     return (size_t)nq * kStageSlots *
@@ -57,8 +74,8 @@ cudaError_t launch_sweep(SweepArgs a, int ndim, int dir, cudaStream_t s) {
     constexpr bool kBoundFp64 = NONUNIF || SIX || ORDER == 3;
     if (dir == 0) {
         const long long total = (long long)(a.g.n[0] + 2) * (a.g.ncell / a.g.n[0]);
-        a.slots_per_block = kStreamSlotsPerBlock;
-        const unsigned blocks = (unsigned)((total + kStreamSlotsPerBlock - 1) / kStreamSlotsPerBlock);
+        a.slots_per_block = stream_slots_per_block(total);
+        const unsigned blocks = (unsigned)((total + a.slots_per_block - 1) / a.slots_per_block);
         if constexpr (LEARNED) {
             switch (ndim) {
                 case 1: sweep_x_stream_learned_kernel<NF, 1><<<blocks, kStreamThreads, 0, s>>>(a); break;
