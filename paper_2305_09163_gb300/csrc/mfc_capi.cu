@@ -112,9 +112,12 @@ bool is_f32(const mfc_ctx* c) { return c->precision != MFC_FP64; }
 
 size_t real_size(const mfc_ctx* c) { return is_f32(c) ? sizeof(float) : sizeof(double); }
 
+bool nonuniform(const mfc_ctx* c) { return c->grid[0] || c->grid[1] || c->grid[2]; }
+
 int auto_segment(const mfc_ctx* c, int dir) {
     if (c->seg_override > 0) return c->seg_override;
-    return sweep_segment(c->ncell, c->n[dir], !is_f32(c) && c->yz_stream != 0);
+    const bool stream = c->six || nonuniform(c) || c->yz_stream != 0;   // the rule of launch_sweep
+    return stream ? stream_segment(c->ncell, c->n[dir], !is_f32(c)) : marching_segment(c->ncell, c->n[dir]);
 }
 
 template <typename F>
@@ -134,8 +137,6 @@ mfc_status launch(mfc_ctx* c, int cat, F&& fn) {
     }
     return MFC_OK;
 }
-
-bool nonuniform(const mfc_ctx* c) { return c->grid[0] || c->grid[1] || c->grid[2]; }
 
 bool has_cbc(const mfc_ctx* c) {
     for (int i = 0; i < 2 * c->ndim; ++i)
@@ -294,7 +295,7 @@ SweepArgs base_sweep(const mfc_ctx* c) {
         a.kpinf[k] = k < c->nf ? c->pi_inf[k] : 0.0;
         a.rc1[k] = k < c->nf ? (c->gamma[k] - 1.0) / c->gamma[k] : 0.0;
     }
-    sweep_set_f32_constants(a);
+    sweep_set_constants(a);
     return a;
 }
 

@@ -131,7 +131,7 @@ __device__ __forceinline__ void kapila_K_df(const SweepArgs& a, const double* w,
     al[NF - 1] = df_from_double(last);
 #pragma unroll
     for (int k = 0; k < NF; ++k)   // gamma_k as float-float: its FP32 rounding would show in K
-        Z[k] = df_mul(df_add(p, df_from_double(a.kpinf[k])), df_from_double(a.kgam[k]));
+        Z[k] = df_mul(df_add(p, a.kpinfd[k]), a.kgamd[k]);
     df pe[NF];   // product of the other phases' Z
 #pragma unroll
     for (int k = 0; k < NF; ++k) {
@@ -230,8 +230,8 @@ __device__ __noinline__ void relax6(const SweepArgs& a, double* q) {
     for (int k = 0; k < NF; ++k) {
         a0d[k] = df_from_double(a0[k]);
         E0d[k] = df_from_double(E0[k]);
-        pid[k] = df_from_double(a.kpinf[k]);
-        c1d[k] = df_from_double(a.rc1[k]);
+        pid[k] = a.kpinfd[k];
+        c1d[k] = a.rc1d[k];
         a0f[k] = a0d[k].hi;
         E0f[k] = E0d[k].hi;
         pif[k] = a.kpinff[k];
@@ -623,10 +623,12 @@ __device__ __forceinline__ void publish_rate(const SweepArgs& a, const RateAcc& 
 }
 
 
-// Finish cell idx (coordinate b along DIR, neighbours sd apart, transverse
-// flat index tr or -1): flux difference and alpha div(u) source, or, at a
-// characteristic boundary, the boundary rate (from cbc_rates when the caller
-// gives tr, else computed here); then store, accumulate or apply the RK stage.
+// Finish cell idx (coordinate b along DIR, neighbours sd apart): flux
+// difference and alpha div(u) source, or, at a characteristic boundary, the
+// boundary rate (from cbc_rates where the caller prepared them, at the cell's
+// transverse index, which is worked out from idx and b there: kept from the
+// start of the sweep it cost the y/z kernels registers; else computed here);
+// then store, accumulate or apply the RK stage.
 //
 // Six-equation model (SIX): NQ rows; the phase energies lose a_k p div(u)
 // (cell values), and an RK stage update ends with the pressure relaxation
@@ -647,7 +649,7 @@ __device__ __forceinline__ void publish_rate(const SweepArgs& a, const RateAcc& 
 // face-velocity divergence.
 template <typename Real, int NF, int NDIM, int DIR, bool SIX = false>
 __device__ __forceinline__ double finish_cell_rates(const SweepArgs& a, long long idx, Real* out, const Real du,
-                                                    const Real* cell, Real inv_dx, int b, long long sd, long long tr,
+                                                    const Real* cell, Real inv_dx, int b, long long sd,
                                                     const unsigned char* stg, int slot) {
     using Lay = Layout<NF, NDIM, SIX>;
     constexpr int NS = Lay::NS, NQ = Lay::NQ, IA = Lay::IA;
@@ -678,7 +680,12 @@ __device__ __forceinline__ double finish_cell_rates(const SweepArgs& a, long lon
         const bool lo = b == 0 && a.g.bc_lo[DIR] == BC_CHARACTERISTIC;
         const bool hi = b == n - 1 && a.g.bc_hi[DIR] == BC_CHARACTERISTIC;
         if (lo || hi) {   // the boundary rate replaces the flux difference and the source
-            if (a.cbc_rates && tr >= 0) {
+            if (a.cbc_rates) {
+                const long long lo_idx = idx - b * sd;   // the row's first cell
+                const long long nx = a.g.n[0];
+                const long long tr = DIR == 0   ? lo_idx / nx
+                                     : DIR == 1 ? lo_idx % nx + nx * (lo_idx / (nx * a.g.n[1]))
+                                                : lo_idx;
                 const Real* rb = static_cast<const Real*>(a.cbc_rates) + a.cbc_off[DIR][lo ? 0 : 1] + tr;
                 const long long nt = a.g.ncell / n;
 #pragma unroll
@@ -765,13 +772,13 @@ __device__ __forceinline__ double finish_cell_rates(const SweepArgs& a, long lon
 template <typename Real, int NF, int NDIM, int DIR, bool SIX = false>
 __device__ __forceinline__ double finish_cell(const SweepArgs& a, long long idx, const Real* Fm, const Real* Fp,
                                               Real um, Real up, const Real* cell, Real inv_dx, int b, long long sd,
-                                              long long tr = -1, const unsigned char* stg = nullptr, int slot = 0) {
+                                              const unsigned char* stg = nullptr, int slot = 0) {
     constexpr int NQ = Layout<NF, NDIM, SIX>::NQ;
     Real out[NQ];
 #pragma unroll
     for (int v = 0; v < NQ; ++v) out[v] = (Fm[v] - Fp[v]) * inv_dx;
     const Real du = (up - um) * inv_dx;
-    return finish_cell_rates<Real, NF, NDIM, DIR, SIX>(a, idx, out, du, cell, inv_dx, b, sd, tr, stg, slot);
+    return finish_cell_rates<Real, NF, NDIM, DIR, SIX>(a, idx, out, du, cell, inv_dx, b, sd, stg, slot);
 }
 
 // Five-equation FP64 path with float-float fluxes: the differences and the
@@ -780,14 +787,13 @@ __device__ __forceinline__ double finish_cell(const SweepArgs& a, long long idx,
 template <int NF, int NDIM, int DIR, bool SIX = false>
 __device__ __forceinline__ double finish_cell_df(const SweepArgs& a, long long idx, const df* Fm, const df* Fp,
                                                  df um, df up, const double* cell, double inv_dx, df inv_df, int b,
-                                                 long long sd, long long tr = -1, const unsigned char* stg = nullptr,
-                                                 int slot = 0) {
+                                                 long long sd, const unsigned char* stg = nullptr, int slot = 0) {
     constexpr int NQ = Layout<NF, NDIM, SIX>::NQ;
     double out[NQ];
 #pragma unroll
     for (int v = 0; v < NQ; ++v) out[v] = df_to_double(df_mul(df_add(Fm[v], df_neg(Fp[v])), inv_df));
     const double du = df_to_double(df_mul(df_add(up, df_neg(um)), inv_df));
-    return finish_cell_rates<double, NF, NDIM, DIR, SIX>(a, idx, out, du, cell, inv_dx, b, sd, tr, stg, slot);
+    return finish_cell_rates<double, NF, NDIM, DIR, SIX>(a, idx, out, du, cell, inv_dx, b, sd, stg, slot);
 }
 
 }  // namespace mfc

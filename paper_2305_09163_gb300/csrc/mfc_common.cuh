@@ -4,6 +4,7 @@
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
+#include <string.h>
 
 #include "mfc_df.cuh"
 #include "mfc_mlp.cuh"
@@ -41,6 +42,35 @@ struct EosConstF {
     float A_N, B_N;
     float dA[2], dB[2];
 };
+
+// The constants of the FP64 path's float-float arithmetic, split once on the
+// host: as kernel arguments they are operands in the constant bank, where split
+// in the kernel they took ~260 instructions of every thread (5% of a CTA that
+// runs one chunk) and registers through the whole sweep.
+struct EosDf {
+    df G_N, P_N, dG[2], dP[2];
+    // six-equation model: the frozen-sound-speed coefficients and the phase
+    // constants G_k = G_N + dG_k, P_k = P_N + dP_k
+    df A_N, B_N, dA[2], dB[2], Gk[2], Pk[2];
+};
+
+// Host: df_from_double, the same bits.
+inline df df_split(double d) {
+    uint64_t u;
+    memcpy(&u, &d, sizeof u);
+    const uint32_t hw = (uint32_t)(u >> 32), lw = (uint32_t)u;
+    const uint32_t sign = hw & 0x80000000u;
+    const int ef = (int)((hw >> 20) & 0x7FFu) - 1023 + 127, es = ef - 52;
+    const uint32_t hb = ef > 0 ? sign | ((uint32_t)ef << 23) | ((hw & 0xFFFFFu) << 3) | (lw >> 29) : 0u;
+    const uint32_t sb = (uint32_t)(es > 1 ? es : 1) << 23;
+    df r;
+    float scale;
+    memcpy(&r.hi, &hb, sizeof hb);
+    memcpy(&scale, &sb, sizeof sb);
+    const float lo = (float)(lw & 0x1FFFFFFFu) * scale;
+    r.lo = es > 0 ? (sign ? -lo : lo) : 0.f;
+    return r;
+}
 
 // Arguments of one directional sweep.
 struct SweepArgs {
@@ -84,10 +114,14 @@ struct SweepArgs {
     float eps34f;
     float epsf;
     float inv_dxf[3];
+    EosDf ed;               // FP64 kernels: e, eps * 3/4, eps and g.inv_dx in float-float
+    df eps34d, epsd, inv_dxd[3];
+    df kgamd[3], kpinfd[3], rc1d[3];   // kgam, kpinf, rc1 in float-float
 };
 
-// Fill the FP32 constants of a from its FP64 ones (host, after e, eps and g).
-inline void sweep_set_f32_constants(SweepArgs& a) {
+// Fill the FP32 and float-float constants of a from its FP64 ones (host, after
+// e, eps, g and the phase constants).
+inline void sweep_set_constants(SweepArgs& a) {
     a.ef.G_N = (float)a.e.G_N;
     a.ef.P_N = (float)a.e.P_N;
     a.ef.A_N = (float)a.e.A_N;
@@ -105,6 +139,26 @@ inline void sweep_set_f32_constants(SweepArgs& a) {
         a.kpinff[k] = (float)a.kpinf[k];
     }
     for (int d = 0; d < 3; ++d) a.inv_dxf[d] = (float)a.g.inv_dx[d];
+    a.ed.G_N = df_split(a.e.G_N);
+    a.ed.P_N = df_split(a.e.P_N);
+    a.ed.A_N = df_split(a.e.A_N);
+    a.ed.B_N = df_split(a.e.B_N);
+    for (int k = 0; k < 2; ++k) {
+        a.ed.dG[k] = df_split(a.e.dG[k]);
+        a.ed.dP[k] = df_split(a.e.dP[k]);
+        a.ed.dA[k] = df_split(a.e.dA[k]);
+        a.ed.dB[k] = df_split(a.e.dB[k]);
+        a.ed.Gk[k] = df_split(a.e.G_N + a.e.dG[k]);
+        a.ed.Pk[k] = df_split(a.e.P_N + a.e.dP[k]);
+    }
+    a.eps34d = df_split(0.75 * a.eps);
+    a.epsd = df_split(a.eps);
+    for (int d = 0; d < 3; ++d) a.inv_dxd[d] = df_split(a.g.inv_dx[d]);
+    for (int k = 0; k < 3; ++k) {
+        a.kgamd[k] = df_split(a.kgam[k]);
+        a.kpinfd[k] = df_split(a.kpinf[k]);
+        a.rc1d[k] = df_split(a.rc1[k]);
+    }
 }
 
 struct PrimArgs {

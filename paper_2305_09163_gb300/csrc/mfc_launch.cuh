@@ -67,7 +67,7 @@ cudaError_t launch_yz_stream(Kernel kernel, unsigned blocks, SweepArgs a, int nq
 // SIX: the six-equation model (stream kernels, WENO5, uniform grids).
 template <typename Real, int NF, bool LEARNED = false, int ORDER = 5, bool NONUNIF = false, bool SIX = false>
 cudaError_t launch_sweep(SweepArgs a, int ndim, int dir, cudaStream_t s) {
-    // FP64 sweeps bounded to 4 CTAs per SM (128 registers, small spills):
+    // FP64 x sweeps bounded to 4 CTAs per SM (128 registers, small spills):
     // faster for the stretched-grid (83.7 -> 71.1 ms per step at 256^3),
     // six-equation (83.4 -> 80.7) and WENO3 (42.1 -> 41.5) variants, slower
     // for the uniform WENO5 ones (61.0 -> 63.8, Kapila 65.3 -> 67.2)
@@ -109,8 +109,8 @@ cudaError_t launch_sweep(SweepArgs a, int ndim, int dir, cudaStream_t s) {
     }
     const int t1 = (dir == 0) ? 1 : 0, t2 = (dir == 2) ? 1 : 2;
     if (NONUNIF || SIX || a.yz_stream) {   // non-uniform grids, six-equation model: the stream kernel only
-        // y/z stream kernel, one CTA per 32 x-lanes of a segment
-        const unsigned blocks = (unsigned)((long long)((a.g.n[t1] + 31) / 32) * a.nseg * a.g.n[t2]);
+        // y/z stream kernel, one CTA per 32 cells of the transverse plane and segment
+        const unsigned blocks = (unsigned)((a.g.ncell / a.g.n[dir] + 31) / 32 * a.nseg);
         auto nq = [](int nd) { return 2 * NF + nd + (SIX ? NF : 0); };
         if constexpr (LEARNED) {
             switch (ndim * 4 + dir) {
@@ -119,14 +119,14 @@ cudaError_t launch_sweep(SweepArgs a, int ndim, int dir, cudaStream_t s) {
                 case 14: return launch_yz_stream<Real, true>(sweep_yz_stream_learned_kernel<NF, 3, 2>, blocks, a, nq(3), s);
                 default: return cudaErrorInvalidValue;
             }
-        } else if constexpr (sizeof(Real) == 8 && kBoundFp64) {
+        } else if constexpr (sizeof(Real) == 8 && (kBoundFp64 || NF <= 2)) {
             switch (ndim * 4 + dir) {
                 case 9: return launch_yz_stream<Real, !NONUNIF>(sweep_yz_stream_f64_kernel<NF, 2, 1, ORDER, NONUNIF, SIX>, blocks, a, nq(2), s);
                 case 13: return launch_yz_stream<Real, !NONUNIF>(sweep_yz_stream_f64_kernel<NF, 3, 1, ORDER, NONUNIF, SIX>, blocks, a, nq(3), s);
                 case 14: return launch_yz_stream<Real, !NONUNIF>(sweep_yz_stream_f64_kernel<NF, 3, 2, ORDER, NONUNIF, SIX>, blocks, a, nq(3), s);
                 default: return cudaErrorInvalidValue;
             }
-        } else if constexpr (sizeof(Real) == 8 && NF == 3 && ORDER == 5) {
+        } else if constexpr (sizeof(Real) == 8) {
             switch (ndim * 4 + dir) {
                 case 9: return launch_yz_stream<Real, true>(sweep_yz_stream_f64b3_kernel<NF, 2, 1>, blocks, a, nq(2), s);
                 case 13: return launch_yz_stream<Real, true>(sweep_yz_stream_f64b3_kernel<NF, 3, 1>, blocks, a, nq(3), s);
@@ -149,9 +149,9 @@ cudaError_t launch_sweep(SweepArgs a, int ndim, int dir, cudaStream_t s) {
             }
         } else {
             switch (ndim * 4 + dir) {
-                case 9: return launch_yz_stream<Real, sizeof(Real) == 8>(sweep_yz_stream_kernel<Real, NF, 2, 1, ORDER, NONUNIF, SIX>, blocks, a, nq(2), s);
-                case 13: return launch_yz_stream<Real, sizeof(Real) == 8>(sweep_yz_stream_kernel<Real, NF, 3, 1, ORDER, NONUNIF, SIX>, blocks, a, nq(3), s);
-                case 14: return launch_yz_stream<Real, sizeof(Real) == 8>(sweep_yz_stream_kernel<Real, NF, 3, 2, ORDER, NONUNIF, SIX>, blocks, a, nq(3), s);
+                case 9: return launch_yz_stream<Real>(sweep_yz_stream_f32_nu_kernel<NF, 2, 1>, blocks, a, nq(2), s);
+                case 13: return launch_yz_stream<Real>(sweep_yz_stream_f32_nu_kernel<NF, 3, 1>, blocks, a, nq(3), s);
+                case 14: return launch_yz_stream<Real>(sweep_yz_stream_f32_nu_kernel<NF, 3, 2>, blocks, a, nq(3), s);
                 default: return cudaErrorInvalidValue;
             }
         }
@@ -256,15 +256,46 @@ inline EosConst make_eos_const(int N, const double* gamma, const double* pi_inf)
     return e;
 }
 
-// Host: cells per thread along direction dir of a sweep.  The FP64 stream
-// sweeps do more work per cell, so longer segments halve the recomputed edge
-// cells (256^3 shock-bubble: 104.4 vs 105.5 ms per step); the length is halved
-// while fewer than ~8 warps per SM would be resident.
-inline int sweep_segment(long long ncell, int n_dir, bool fp64_stream) {
+// Host: cells per thread along direction dir of a marching sweep; halved while
+// fewer than ~8 warps per SM would be resident.
+inline int marching_segment(long long ncell, int n_dir) {
     const long long trans = ncell / n_dir;
-    int L = fp64_stream ? 128 : 64;
+    int L = 64;
     while (L > 8 && trans * ((n_dir + L - 1) / L) < 152LL * 4 * kSweepThreads) L /= 2;
     return L;
+}
+
+// Host: cells per segment of a y/z stream sweep.  A segment of L cells walks
+// ceil((L + 2)/4) chunks of 4 edge cells, two of which a neighbour repeats, so
+// only lengths 4 m - 2 (and what is left at the end) are taken: 128 cells took
+// 33 chunks for the work of 32.5.  Long segments repeat fewer cells, short ones
+// fill the chip, so the length with the smallest estimate is taken, in units of
+// the time an SM with all its CTAs spends per chunk:
+//     chunks of all CTAs / 152 SMs  +  tail * chunks of one CTA,
+// each CTA charged a quarter of a chunk for its first rows.  The tail is what a
+// CTA's walk adds when it does not overlap others: an SM holds 4 FP64 CTAs, and
+// one alone takes 7.5 us per chunk where four share it at 4.15 us each; it holds
+// 8 FP32 ones, 2.1 us against 0.55 us.  Measured over lengths 8-254 the estimate's
+// choice is within 5% of the best one: FP64 y sweep of 64^3 97 -> 82 us, 100x90x77
+// 234 -> 182, 600x500 98 -> 87, 128^3 577 -> 504, 256^3 3.76 -> 3.69 ms, against
+// the former rule (lengths halved from 128 or 64 until ~8 warps per SM had work).
+inline int stream_segment(long long ncell, int n_dir, bool fp64) {
+    const long long columns = (ncell / n_dir + 31) / 32;
+    const double tail = fp64 ? 1.0 : 2.5, start = 0.25;
+    int best = n_dir;
+    double least = 0.0;
+    for (int L = 2;; L += 4) {
+        const int whole = n_dir / L, rest = n_dir % L;
+        const double walk = (L + 2) / 4 + start;
+        const double all = (whole * walk + (rest ? (rest + 5) / 4 + start : 0.0)) * (double)columns;
+        const double t = all / 152.0 + tail * walk;
+        if (L == 2 || t < least) {
+            least = t;
+            best = L;
+        }
+        if (L >= n_dir) break;
+    }
+    return best;
 }
 
 // Explicitly instantiated in the mfc_inst_*.cu units.

@@ -93,8 +93,8 @@ cudaError_t run(const Geometry& g, const EosConst& e, int ndim, const double* q,
         a.fallback = fallback;
         a.fallback_count = nullptr;
         a.cbc = cbc;
-        sweep_set_f32_constants(a);
-        a.seg = sweep_segment(g.ncell, g.n[d], true);
+        sweep_set_constants(a);
+        a.seg = stream_segment(g.ncell, g.n[d], true);
         a.nseg = (g.n[d] + a.seg - 1) / a.seg;
         rc = launch_sweep<double, NF>(a, ndim, d, s);
         if (rc != cudaSuccess) return rc;

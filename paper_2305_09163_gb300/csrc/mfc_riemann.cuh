@@ -306,28 +306,6 @@ __device__ __forceinline__ void hllc_df(const double* L, const double* R, const 
     }
 }
 
-// The EOS constants as float-float values (split once per kernel).
-struct EosDf {
-    df G_N, P_N, dG[2], dP[2];
-    // six-equation model: the frozen-sound-speed coefficients and the phase
-    // constants G_k = G_N + dG_k, P_k = P_N + dP_k
-    df A_N, B_N, dA[2], dB[2], Gk[2], Pk[2];
-    template <typename E>
-    __device__ __forceinline__ explicit EosDf(const E& e)
-        : G_N(df_from_double((double)e.G_N)), P_N(df_from_double((double)e.P_N)),
-          A_N(df_from_double((double)e.A_N)), B_N(df_from_double((double)e.B_N)) {
-#pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            dG[k] = df_from_double((double)e.dG[k]);
-            dP[k] = df_from_double((double)e.dP[k]);
-            dA[k] = df_from_double((double)e.dA[k]);
-            dB[k] = df_from_double((double)e.dB[k]);
-            Gk[k] = df_from_double((double)e.G_N + (double)e.dG[k]);
-            Pk[k] = df_from_double((double)e.P_N + (double)e.dP[k]);
-        }
-    }
-};
-
 // Mixture quantities of a float-float face state, in float-float (SIX: n =
 // Gamma r c^2 with the frozen sound speed, r c^2 = A p + B, as in mixture).
 template <int NF, int NDIM, bool SIX = false>
@@ -447,10 +425,11 @@ __device__ __forceinline__ void face_flux(const SweepArgs& a, const EosR<Real>& 
 // phase N is a trace (alpha_N ~ 1e-6) the subtraction cancels and a
 // float-float alpha_k (~2^-48 of 1) would leave alpha_N ~3e-9 relative error.
 template <int NF, int NDIM, int DIR, bool SIX = false>
-__device__ __forceinline__ void face_flux_df(const SweepArgs& a, const EosDf& e, const df* eLs, const df* eRs,
+__device__ __forceinline__ void face_flux_df(const SweepArgs& a, const df* eLs, const df* eRs,
                                              const double* cl, const double* cr, df* F, df& ut) {
     using Lay = Layout<NF, NDIM>;
     constexpr int NS = Lay::NS;
+    const EosDf& e = a.ed;
     df sl[NS], sr[NS];
     [[maybe_unused]] double aL[SIX ? NF - 1 : 1], aR[SIX ? NF - 1 : 1];
 #pragma unroll

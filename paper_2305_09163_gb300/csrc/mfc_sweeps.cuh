@@ -174,16 +174,16 @@ __global__ void __launch_bounds__(128) sweep_kernel(const SweepArgs a) {
 // ---------------------------------------------------------------------------
 template <typename Real, int NF, int NDIM, int ORDER, bool NONUNIF, bool SIX, bool VALUE_MAJOR>
 __device__ __forceinline__ void dfs_edges(const SweepArgs& a, int dir, int c, int q, double vc, const double (&D)[4],
-                                          double eps34, df& eR, df& eL) {
+                                          df& eR, df& eL) {
     df2 I;
     if constexpr (NONUNIF) {
         const GridCol<VALUE_MAJOR> grow(a.grid[dir], a.grid_stride[dir], c);
-        I = weno5_increments_nu_pair(D, sweep_epsw<double, 3>(a), grow);
+        I = weno5_increments_nu_pair(D, a.epsd, grow);
     } else if constexpr (ORDER == 5) {
         const df d[4] = {df_from_double(D[0]), df_from_double(D[1]), df_from_double(D[2]), df_from_double(D[3])};
-        I = weno5_increments_pair(d, eps34);
+        I = weno5_increments_pair(d, a.eps34d);
     } else {
-        I = weno3_increments_pair(D[1], D[2], eps34);
+        I = weno3_increments_pair(D[1], D[2], a.epsd);
     }
     if (SIX && q >= Layout<NF, NDIM>::IA && q < Layout<NF, NDIM>::IA + NF - 1) {
         eL = df_pack(vc + df_to_double(df2_x(I)));
@@ -245,9 +245,7 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
     const int bclo = a.g.bc_lo[0], bchi = a.g.bc_hi[0];
     const Real eps34 = sweep_epsw<Real, ORDER>(a);  // 3/4 eps (WENO5) or eps (WENO3)
     const EosR<Real> e = sweep_eos<Real>(a);
-    [[maybe_unused]] const EosDf edf(e);   // DFS: the EOS constants as float-float
     const Real inv_dx = sweep_inv_dx<Real>(a, 0);
-    [[maybe_unused]] const df inv_df = df_from_double((double)inv_dx);
     const int t = threadIdx.x;
     LearnRows* lsm = nullptr;
     if constexpr (LEARNED) {
@@ -349,7 +347,7 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
                 Dv[q][0] = Dv[q][1] = Dv[q][2] = Dv[q][3] = 0;
             }
         }
-        if (ROLL && live) {
+        if constexpr (ROLL) if (live) {
             int mk[5];
             bool fk[5];
 #pragma unroll
@@ -373,22 +371,10 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
                     for (int k = 0; k < 5; ++k) vn[k] = __ldg(wr + (q + 1) * nc + mk[k]);
                 }
                 Real Dq[4] = {v[1] - v[0], v[2] - v[1], v[3] - v[2], v[4] - v[3]};
-                if constexpr (DFS) {
-                    df er, el;
-                    dfs_edges<Real, NF, NDIM, ORDER, NONUNIF, SIX, true>(a, 0, c, q, v[2], Dq, eps34, er, el);
-                    dsh_eL[q][pos] = el;
-                    dsh_eR[q][t] = er;
-                } else {
-                    Real er, el;
-                    if constexpr (NONUNIF) {
-                        const GridCol<true> grow(a.grid[0], a.grid_stride[0], c);
-                        weno5_edges_nu(v[2], Dq, sweep_epsw<Real, 3>(a), grow, er, el);
-                    } else {
-                        weno_edges<ORDER>(v[2], Dq, eps34, er, el);
-                    }
-                    sh_eL[q][pos] = el;
-                    sh_eR[q][t] = er;
-                }
+                df er, el;
+                dfs_edges<Real, NF, NDIM, ORDER, NONUNIF, SIX, true>(a, 0, c, q, v[2], Dq, er, el);
+                dsh_eL[q][pos] = el;
+                dsh_eR[q][t] = er;
             }
 #pragma unroll
             for (int q = 0; q < NS; ++q) {
@@ -397,7 +383,7 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
                 vcv[q] = (q == IM && fk[2]) ? -x2 : x2;
             }
         }
-        if (!ROLL && !LEARNED && live) {
+        if constexpr (!ROLL && !LEARNED) if (live) {
             Real v[5][NS];
 #pragma unroll
             for (int k = 0; k < 5; ++k) {
@@ -417,7 +403,7 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
                 cm1[q] = v[1][q];
             }
         }
-        if (!ROLL && !LEARNED && live) {
+        if constexpr (!ROLL && !LEARNED) if (live) {
             if constexpr (NONUNIF) {
                 const GridCol<true> row(a.grid[0], a.grid_stride[0], c);
                 const Real epsn = sweep_epsw<Real, 3>(a);   // unscaled eps
@@ -434,7 +420,7 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
         }
         // left-side values of this chunk (the last chunk's last slot stays at
         // the position before this chunk's first)
-        if (!ROLL && !LEARNED && live) {
+        if constexpr (!ROLL && !LEARNED) if (live) {
 #pragma unroll
             for (int q = 0; q < NS; ++q) sh_eL[q][pos] = eL[q];
         }
@@ -450,7 +436,7 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
                 lftd[q] = dsh_eL[q][pl];
                 erd[q] = dsh_eR[q][t];
             }
-            face_flux_df<NF, NDIM, 0, SIX>(a, edf, lftd, erd, cm1, cell, Fd, utd);
+            face_flux_df<NF, NDIM, 0, SIX>(a, lftd, erd, cm1, cell, Fd, utd);
 #pragma unroll
             for (int q = 0; q < NQ; ++q) dsh_F[q][pos] = Fd[q];
             dsh_F[NQ][pos] = utd;
@@ -488,13 +474,13 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) Fm[q] = dsh_F[q][pl];
                 double idx_d = inv_dx;
-                df idx_df = inv_df;
+                df idx_df = a.inv_dxd[0];
                 if constexpr (NONUNIF) {   // this cell's width
                     idx_df = grid_df(GridCol<true>(a.grid[0], a.grid_stride[0], c - 1), kGridInvDx);
                     idx_d = df_to_double(idx_df);
                 }
                 racc.add(finish_cell_df<NF, NDIM, 0, SIX>(a, rowoff + (c - 1), Fm, Fd, dsh_F[NQ][pl], utd, cm1, idx_d,
-                                                     idx_df, c - 1, 1, row));
+                                                     idx_df, c - 1, 1));
             }
         } else if (has_face && s >= own0 && c >= 1) {
             Real Fm[NQ];
@@ -502,7 +488,7 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
             for (int q = 0; q < NQ; ++q) Fm[q] = sh_F[q][pl];
             racc.add(finish_cell<Real, NF, NDIM, 0, SIX>(
                 a, rowoff + (c - 1), Fm, F, sh_F[NQ][pl], ut, cm1,
-                NONUNIF ? grid_inv_dx<true>(a.grid[0], a.grid_stride[0], c - 1, Real(0)) : inv_dx, c - 1, 1, row));
+                NONUNIF ? grid_inv_dx<true>(a.grid[0], a.grid_stride[0], c - 1, Real(0)) : inv_dx, c - 1, 1));
         }
         // No barrier is needed here: the next chunk writes edge values
         // (position pl of this chunk) after this chunk's second barrier, which
@@ -554,7 +540,8 @@ __global__ void __launch_bounds__(kStreamThreads, 4) sweep_x_stream_f64_kernel(c
 
 // ---------------------------------------------------------------------------
 // y or z sweep as a coalesced stream.  A CTA of 4 warps covers 32
-// consecutive x (lanes) of one pencil segment s0..s1-1 along DIR and walks it
+// consecutive cells (lanes) of the transverse plane, x fastest, of one pencil
+// segment s0..s1-1 along DIR and walks it
 // in chunks of 4 edge cells, one per warp: warp r of a chunk reconstructs the
 // edges of cell c = base + r from its five-cell stencil, read from a shared
 // ring of the 8 rows base-2..base+5 (each warp loads one new row per chunk,
@@ -581,8 +568,6 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
     constexpr int NS = Lay::NS, IM = Lay::IM;
     constexpr int NQ = Layout<NF, NDIM, SIX>::NQ;   // flux rows
     constexpr int NJ = LEARNED ? NS : 1;
-    constexpr int T1 = 0;
-    constexpr int T2 = (DIR == 2) ? 1 : 2;
     constexpr int RING = 2 * kRowsPerChunk;  // rows base-2 .. base+5 of a chunk
     // Edge values and face fluxes of cell c sit in row c mod ER of a ring of
     // ER = kRowsPerChunk + 1 rows: a chunk writes its four cells and reads
@@ -607,27 +592,29 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
     static_assert(32 * kRowsPerChunk == kStageSlots, "one staging slot per thread");
     const Real* __restrict__ w = static_cast<const Real*>(a.w);
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
-    const int n1 = a.g.n[T1], n2 = a.g.n[T2], nd = a.g.n[DIR];
-    const int nxc = (n1 + 31) >> 5;
-    const long long bid = blockIdx.x;
-    const int xc = (int)(bid % nxc);
-    const long long rest = bid / nxc;
-    const int sg = (int)(rest % a.nseg);
-    const int t2 = (int)(rest / a.nseg);
-    if (t2 >= n2) return;  // whole CTA
-    const bool active = xc * 32 + lane < n1;
-    const int t1 = active ? xc * 32 + lane : n1 - 1;
-    const long long sd = stride_of(a.g, DIR);
-    const long long basei = (long long)t1 * stride_of(a.g, T1) + (long long)t2 * stride_of(a.g, T2);
+    // lanes run over the flat transverse plane (x fastest), so only the plane's
+    // last warp has idle lanes, whatever the row length
+    const int nd = a.g.n[DIR];
+    // 32-bit indices (registers): 2D and 3D states take at least 112 bytes per
+    // cell, so the device's memory holds fewer than 2^32 cells and, of three
+    // planes or rows at least, fewer than 2^31 in one
+    const int plane = (int)(a.g.ncell / nd);
+    const int ncol = (plane + 31) >> 5;
+    const int sg = (int)(blockIdx.x / (unsigned)ncol);
+    const int flat = ((int)blockIdx.x - sg * ncol) * 32 + lane;
+    const bool active = flat < plane;
+    const int tr = active ? flat : plane - 1;
+    const unsigned sd = (unsigned)stride_of(a.g, DIR);
+    // z: the plane is contiguous; y: rows of n[0] cells, a plane of n[0] n[1] apart
+    const int n0 = a.g.n[0];
+    const unsigned basei = DIR == 2 ? (unsigned)tr : (unsigned)(tr % n0) + (unsigned)(tr / n0) * ((unsigned)n0 * (unsigned)a.g.n[1]);
     const long long nc = a.g.ncell;
     const int s0 = sg * a.seg;
     const int s1 = min(s0 + a.seg, nd);
     const int bclo = a.g.bc_lo[DIR], bchi = a.g.bc_hi[DIR];
     const Real eps34 = sweep_epsw<Real, ORDER>(a);  // 3/4 eps (WENO5) or eps (WENO3)
     const EosR<Real> e = sweep_eos<Real>(a);
-    [[maybe_unused]] const EosDf edf(e);   // DFS: the EOS constants as float-float
     const Real inv_dx = sweep_inv_dx<Real>(a, DIR);
-    [[maybe_unused]] const df inv_df = df_from_double((double)inv_dx);
     LearnRows* lsm = nullptr;
     if constexpr (LEARNED) {
         __shared__ LearnRows lbuf[kRowsPerChunk];
@@ -639,7 +626,7 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
     auto load = [&](int i, Real* out) {
         bool flip = false;
         const int m = ghost_map(i, nd, bclo, bchi, &flip);
-        const long long idx = basei + (long long)m * sd;
+        const long long idx = basei + (unsigned)m * sd;
 #pragma unroll
         for (int q = 0; q < NS; ++q) out[q] = __ldg(w + q * nc + idx);
         if (flip) out[IM + DIR] = -out[IM + DIR];
@@ -669,7 +656,7 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
         const bool live = c <= s1;
         const bool fin = live && c >= s0 + 1 && active;   // this lane finishes cell c-1 in this chunk
         if (fin) {
-            const long long fidx = basei + (long long)(c - 1) * sd;
+            const long long fidx = basei + (unsigned)(c - 1) * sd;
             int staged = 0;
             if constexpr (STAGE) {
                 staged = a.stage;
@@ -713,22 +700,10 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
                     const Real v0 = ring[s0r][q][lane], v1 = ring[s1r][q][lane], v2 = ring[s2r][q][lane];
                     const Real v3 = ring[s3r][q][lane], v4 = ring[s4r][q][lane];
                     Real Dq[4] = {v1 - v0, v2 - v1, v3 - v2, v4 - v3};
-                    if constexpr (DFS) {
-                        df er, el;
-                        dfs_edges<Real, NF, NDIM, ORDER, NONUNIF, SIX, false>(a, DIR, c, q, v2, Dq, eps34, er, el);
-                        dsh_eL[q][eslot(c)][lane] = el;
-                        dsh_eR[q][row][lane] = er;
-                    } else {
-                        Real er, el;
-                        if constexpr (NONUNIF) {
-                            const GridCol<false> grow(a.grid[DIR], a.grid_stride[DIR], c);
-                            weno5_edges_nu(v2, Dq, sweep_epsw<Real, 3>(a), grow, er, el);
-                        } else {
-                            weno_edges<ORDER>(v2, Dq, eps34, er, el);
-                        }
-                        sh_eL[q][eslot(c)][lane] = el;
-                        sh_eR[q][row][lane] = er;
-                    }
+                    df er, el;
+                    dfs_edges<Real, NF, NDIM, ORDER, NONUNIF, SIX, false>(a, DIR, c, q, v2, Dq, er, el);
+                    dsh_eL[q][eslot(c)][lane] = el;
+                    dsh_eR[q][row][lane] = er;
                 }
 #pragma unroll
                 for (int q = 0; q < NS; ++q) {
@@ -781,7 +756,7 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
                 lftd[q] = dsh_eL[q][eslot(c - 1)][lane];
                 erd[q] = dsh_eR[q][row][lane];
             }
-            face_flux_df<NF, NDIM, DIR, SIX>(a, edf, lftd, erd, cm1, cell, Fd, utd);
+            face_flux_df<NF, NDIM, DIR, SIX>(a, lftd, erd, cm1, cell, Fd, utd);
 #pragma unroll
             for (int q = 0; q < NQ; ++q) dsh_F[q][eslot(c)][lane] = Fd[q];
             dsh_F[NQ][eslot(c)][lane] = utd;
@@ -826,22 +801,22 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) Fm[q] = dsh_F[q][eslot(c - 1)][lane];
                 double idx_d = inv_dx;
-                df idx_df = inv_df;
+                df idx_df = a.inv_dxd[DIR];
                 if constexpr (NONUNIF) {   // this cell's width
                     idx_df = grid_df(GridCol<false>(a.grid[DIR], a.grid_stride[DIR], c - 1), kGridInvDx);
                     idx_d = df_to_double(idx_df);
                 }
-                racc.add(finish_cell_df<NF, NDIM, DIR, SIX>(a, basei + (long long)(c - 1) * sd, Fm, Fd,
+                racc.add(finish_cell_df<NF, NDIM, DIR, SIX>(a, basei + (unsigned)(c - 1) * sd, Fm, Fd,
                                                        dsh_F[NQ][eslot(c - 1)][lane], utd, cm1, idx_d, idx_df, c - 1,
-                                                       sd, (long long)t1 + (long long)n1 * t2, stg, threadIdx.x));
+                                                       sd, stg, threadIdx.x));
             } else {
                 Real Fm[NQ];
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) Fm[q] = sh_F[q][eslot(c - 1)][lane];
                 racc.add(finish_cell<Real, NF, NDIM, DIR, SIX>(
-                    a, basei + (long long)(c - 1) * sd, Fm, F, sh_F[NQ][eslot(c - 1)][lane], ut, cm1,
+                    a, basei + (unsigned)(c - 1) * sd, Fm, F, sh_F[NQ][eslot(c - 1)][lane], ut, cm1,
                     NONUNIF ? grid_inv_dx<false>(a.grid[DIR], a.grid_stride[DIR], c - 1, Real(0)) : inv_dx, c - 1, sd,
-                    (long long)t1 + (long long)n1 * t2, stg, threadIdx.x));
+                    stg, threadIdx.x));
             }
         }
         // No barrier is needed here: the next chunk writes edge values (row
@@ -855,21 +830,20 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
     publish_rate(a, racc);
 }
 
-// The y/z stream kernel (FP64 uniform WENO5 forms, with staged finish
-// operands, and the mixed form on non-uniform grids, without: staging took
-// it from 96 to 123 registers): the compiler's own register allocation.
-template <typename Real, int NF, int NDIM, int DIR, int ORDER = 5, bool NONUNIF = false, bool SIX = false>
-__global__ void __launch_bounds__(32 * kRowsPerChunk) sweep_yz_stream_kernel(const SweepArgs a) {
-    sweep_yz_stream_body<Real, NF, NDIM, DIR, false, ORDER, NONUNIF, SIX, sizeof(Real) == 8>(a);
+// The mixed form's y/z stream kernel on non-uniform grids: the compiler's own
+// register allocation, no staging (it took the kernel from 96 to 123 registers).
+template <int NF, int NDIM, int DIR>
+__global__ void __launch_bounds__(32 * kRowsPerChunk) sweep_yz_stream_f32_nu_kernel(const SweepArgs a) {
+    sweep_yz_stream_body<float, NF, NDIM, DIR, false, 5, true>(a);
 }
 
 // The mixed form's five-equation y/z stream kernel on uniform grids, with
-// staged finish operands: bounded to 8 CTAs per SM for up to two fluids (64
-// registers, no spills), 5 for three, so that the registers allow the
-// residency the staging's shared memory does.  The learned form gets its own
-// entry below.
+// staged finish operands: bounded to 7 CTAs per SM for up to two fluids (72
+// registers; 256^3 y / z sweep 499 / 751 us, at 8 CTAs and 64 registers 44-48
+// bytes of spills and 513 / 791, at 6 CTAs 509 / 808), 5 for three.  The learned
+// form gets its own entry below.
 template <int NF, int NDIM, int DIR, int ORDER = 5>
-__global__ void __launch_bounds__(32 * kRowsPerChunk, NF <= 2 ? 8 : 5) sweep_yz_stream_f32_kernel(const SweepArgs a) {
+__global__ void __launch_bounds__(32 * kRowsPerChunk, NF <= 2 ? 7 : 5) sweep_yz_stream_f32_kernel(const SweepArgs a) {
     sweep_yz_stream_body<float, NF, NDIM, DIR, false, ORDER, false, false, true>(a);
 }
 
@@ -882,9 +856,11 @@ __global__ void __launch_bounds__(32 * kRowsPerChunk, 5) sweep_yz_stream_six32_k
     sweep_yz_stream_body<float, NF, NDIM, DIR, false, ORDER, NONUNIF, true, true>(a);
 }
 
-// The bounded FP64 y/z stream kernel (stretched-grid, six-equation and WENO3
-// forms, 4 CTAs per SM).  Staging pays for WENO3 (40.7 -> 39.2 ms per step at
-// 256^3), not on stretched grids (70.0 -> 71.8 ms, more spills at the bound).
+// The FP64 y/z stream kernel, bounded to 4 CTAs per SM (128 registers; the
+// uniform WENO5 form fits without spills and takes 138, one CTA fewer, when left
+// unbounded: 256^3 y sweep 3.76 against 3.42 ms).  Staging pays
+// for WENO3 (40.7 -> 39.2 ms per step at 256^3), not on stretched grids (70.0 ->
+// 71.8 ms, more spills at the bound).
 template <int NF, int NDIM, int DIR, int ORDER = 5, bool NONUNIF = false, bool SIX = false>
 __global__ void __launch_bounds__(32 * kRowsPerChunk, 4) sweep_yz_stream_f64_kernel(const SweepArgs a) {
     sweep_yz_stream_body<double, NF, NDIM, DIR, false, ORDER, NONUNIF, SIX, !NONUNIF>(a);

@@ -42,14 +42,13 @@ namespace mfc {
 // stencil's differences, far inside the path's parity tolerance; scalings by
 // powers of two are exact.  (256^3 FP64 step: 39.0 -> 35.9 ms against the same
 // arithmetic in scalar FP32 instructions.)
-__device__ __forceinline__ df2 weno5_increments_pair(const df (&D)[4], double eps34) {
+__device__ __forceinline__ df2 weno5_increments_pair(const df (&D)[4], df e) {
     const df2 X0 = df2_make(D[0], df_neg(D[3])), X1 = df2_make(D[1], df_neg(D[2]));
     const df2 X2 = df2_swap(df2_neg(X1)), X3 = df2_swap(df2_neg(X0));   // (D2, -D1), (D3, -D0)
     const df2 SX1 = df2_mul(X1, X1);                                     // (D1^2, D2^2)
     const df2 B = df2_add_fast(df2_add_fast(df2_mul(X0, X0), df2_mul_f(df2_mul(X1, X0), f2(-2.75f))),
                                df2_mul_f(SX1, f2(2.5f)));                // (b0, b2)
     const df b1 = df_add_fast(df_add_fast(df2_x(SX1), df2_y(SX1)), df_mul_f(df_mul(D[1], D[2]), -1.25f));
-    const df e = df_from_double(eps34);
     const df2 T = df2_add_fast(df2_make(e, e), B);                       // (t0, t2)
     const df t1 = df_add_fast(e, b1);
     const float m = fminf(T.hi.x, fminf(t1.hi, T.hi.y));
@@ -67,7 +66,7 @@ __device__ __forceinline__ df2 weno5_increments_pair(const df (&D)[4], double ep
     return df2_div(num, den);   // (increment at c+1/2, increment at c-1/2)
 }
 
-__device__ __forceinline__ void weno5_increments_df(const df (&D)[4], double eps34, df& iR, df& iL) {
+__device__ __forceinline__ void weno5_increments_df(const df (&D)[4], df eps34, df& iR, df& iL) {
     const df2 I = weno5_increments_pair(D, eps34);
     iL = df2_x(I);
     iR = df2_y(I);
@@ -75,7 +74,7 @@ __device__ __forceinline__ void weno5_increments_df(const df (&D)[4], double eps
 
 __device__ __forceinline__ void weno5_increments(const double D[4], double eps34, df& iR, df& iL) {
     const df d[4] = {df_from_double(D[0]), df_from_double(D[1]), df_from_double(D[2]), df_from_double(D[3])};
-    weno5_increments_df(d, eps34, iR, iL);
+    weno5_increments_df(d, df_from_double(eps34), iR, iL);
 }
 
 // The two edge values in FP64 (the increments widened and added to v_c).
@@ -141,8 +140,8 @@ __device__ __forceinline__ void weno5_edges(float vc, const float D[4], float ep
 // ---------------------------------------------------------------------------
 // The two WENO3 increments (c+1/2 in lane x, c-1/2 in lane y): lane y evaluates
 // the c+1/2 formula on the mirrored differences (-b, -a).
-__device__ __forceinline__ df2 weno3_increments_pair(double a, double b, double eps) {
-    const df A = df_from_double(a), Bd = df_from_double(b), E = df_from_double(eps);
+__device__ __forceinline__ df2 weno3_increments_pair(double a, double b, df E) {
+    const df A = df_from_double(a), Bd = df_from_double(b);
     const df2 X = df2_make(A, df_neg(Bd)), Y = df2_make(Bd, df_neg(A));
     const df2 T = df2_add_fast(df2_make(E, E), df2_mul(df2_make(A, Bd), df2_make(A, Bd)));   // (t0, t1)
     const float m = fminf(T.hi.x, T.hi.y);
@@ -154,7 +153,7 @@ __device__ __forceinline__ df2 weno3_increments_pair(double a, double b, double 
     return df2_div(num, den);
 }
 __device__ __forceinline__ void weno3_edges(double vc, double a, double b, double eps, double& eR, double& eL) {
-    const df2 I = weno3_increments_pair(a, b, eps);
+    const df2 I = weno3_increments_pair(a, b, df_from_double(eps));
     eL = vc + df_to_double(df2_x(I));
     eR = vc + df_to_double(df2_y(I));
 }
@@ -197,7 +196,7 @@ __device__ __forceinline__ df grid_df(const Col& row, int k) {
 }
 
 template <class Col>
-__device__ __forceinline__ df2 weno5_increments_nu_pair(const double D[4], double eps, const Col& row) {
+__device__ __forceinline__ df2 weno5_increments_nu_pair(const double D[4], df e, const Col& row) {
     // the two edges side by side in packed FP32 instructions: lane x the c+1/2
     // edge (coefficients 0-5, 12-14), lane y the c-1/2 edge (6-11, 15-17); the
     // smoothness indicators b0 and b2 side by side, b1 alone
@@ -211,7 +210,6 @@ __device__ __forceinline__ df2 weno5_increments_nu_pair(const double D[4], doubl
                                df2_mul(C(20, 26), Shi));           // (b0, b2)
     const df b1 = df_add_fast(df_add_fast(df_mul(grid_df(row, 21), df2_x(Shi)), df_mul(grid_df(row, 22), df_mul(d1, d2))),
                               df_mul(grid_df(row, 23), df2_y(Slo)));
-    const df e = df_from_double(eps);
     const df2 T = df2_add_fast(df2_make(e, e), B);                 // (t0, t2)
     const df t1 = df_add_fast(e, b1);
     const float m = fminf(T.hi.x, fminf(t1.hi, T.hi.y));
@@ -228,13 +226,6 @@ __device__ __forceinline__ df2 weno5_increments_nu_pair(const double D[4], doubl
     const df2 num = df2_add_fast(df2_add_fast(df2_mul(W0, P0), df2_mul(W1, P1)), df2_mul(W2, P2));
     const df2 den = df2_add_fast(df2_add_fast(W0, W1), W2);
     return df2_div(num, den);   // (increment at c+1/2, increment at c-1/2)
-}
-template <class Col>
-__device__ __forceinline__ void weno5_edges_nu(double vc, const double D[4], double eps, const Col& row,
-                                               double& eR, double& eL) {
-    const df2 I = weno5_increments_nu_pair(D, eps, row);
-    eL = vc + df_to_double(df2_x(I));
-    eR = vc + df_to_double(df2_y(I));
 }
 template <class Col>
 __device__ __forceinline__ void weno5_edges_nu(float vc, const float D[4], float eps, const Col& row,

@@ -32,3 +32,12 @@ def _check(n, bc=1, nf=2, **params):
 @pytest.mark.parametrize("n", [(124,), (125,), (250,), (1000,), (40, 3), (61, 7), (5, 200), (1021, 400)])
 def test_x_share_edges(n):
     _check(n)
+
+
+# y/z CTAs take 32 cells of the flat transverse plane and segments of 4 m - 2
+# cells: planes of 15, 32, 33 and 31 cells, directions that leave 1, 2 or 3 cells
+# to the last segment, 2D rows below, at and above a warp
+@pytest.mark.parametrize("n", [(5, 3, 3), (8, 4, 8), (11, 7, 3), (31, 131, 3), (3, 3, 77), (31, 9), (32, 127), (33, 130)])
+@pytest.mark.parametrize("bc", [0, 2, 3])
+def test_yz_plane_and_segment_edges(n, bc):
+    _check(n, bc)
