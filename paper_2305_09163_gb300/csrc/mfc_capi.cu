@@ -251,8 +251,17 @@ mfc_status ensure_alive(mfc_ctx* c) {
     return MFC_OK;
 }
 
-// Primitive recovery of src into c->w (optionally with the CFL rate).
-mfc_status run_prims(mfc_ctx* c, const double* src, bool rate) {
+cudaError_t dispatch_relax_prims(const mfc_ctx* c, const PrimArgs& a, bool rate) {
+    const RelaxConst k = make_relax_const(c->nf, c->gamma, c->pi_inf, c->e);
+    if (is_f32(c)) return c->nf == 2 ? launch_relax_prims<float, 2>(a, k, c->ndim, rate, c->stream)
+                                     : launch_relax_prims<float, 3>(a, k, c->ndim, rate, c->stream);
+    return c->nf == 2 ? launch_relax_prims<double, 2>(a, k, c->ndim, rate, c->stream)
+                      : launch_relax_prims<double, 3>(a, k, c->ndim, rate, c->stream);
+}
+
+// Primitive recovery of src into c->w (optionally with the CFL rate); relax:
+// six-equation model, src is first relaxed in place.
+mfc_status run_prims(mfc_ctx* c, const double* src, bool rate, bool relax = false) {
     PrimArgs a{};
     a.g = c->g;
     a.e = c->e;
@@ -264,7 +273,8 @@ mfc_status run_prims(mfc_ctx* c, const double* src, bool rate) {
         a.grid[d] = c->grid[d];
         a.grid_stride[d] = c->n[d] + 2;
     }
-    return launch(c, rate ? P_CFL : P_PRIMS, [&] { return dispatch_prims(c, a, rate); });
+    return launch(c, rate ? P_CFL : P_PRIMS,
+                  [&] { return relax ? dispatch_relax_prims(c, a, rate) : dispatch_prims(c, a, rate); });
 }
 
 SweepArgs base_sweep(const mfc_ctx* c) {
@@ -293,7 +303,6 @@ SweepArgs base_sweep(const mfc_ctx* c) {
     for (int k = 0; k < 3; ++k) {
         a.kgam[k] = k < c->nf ? c->gamma[k] : 1.0;
         a.kpinf[k] = k < c->nf ? c->pi_inf[k] : 0.0;
-        a.rc1[k] = k < c->nf ? (c->gamma[k] - 1.0) / c->gamma[k] : 0.0;
     }
     sweep_set_constants(a);
     return a;
@@ -712,21 +721,25 @@ mfc_status mfc_step(mfc_ctx* c, double dt) {
     // primitives of the stage's new state into w2 (then swapped with w), and
     // the last stage also the CFL rate of q^{n+1}, so no separate recovery pass
     // runs (256^3 shock-bubble: 59.0 -> 58.2 ms per step).  The six-equation
-    // model relaxes in the epilogue and the FP32 forms' memory-bound z sweep
-    // gains nothing from it: they recover separately.
+    // model relaxes every stage's state in a pass of its own, which recovers
+    // the primitives and, in the last stage, the CFL rate too.  The FP32 forms'
+    // memory-bound z sweep gains nothing from a fused recovery: they recover
+    // separately.
     const bool fused = !c->six && !is_f32(c);
     auto stage = [&](const RkStage& st, bool last) -> mfc_status {
-        if (!fused) return run_sweeps(c, nullptr, &st);
-        if (last) {
+        if (last && (fused || c->six)) {
             MFC_CUDA(c, cudaMemsetAsync(c->d_rate, 0, sizeof(unsigned long long), c->stream));
             MFC_CUDA(c, cudaMemsetAsync(c->d_bad, 0, sizeof(int), c->stream));
         }
-        mfc_status r = run_sweeps(c, nullptr, &st, c->w2, last);
+        mfc_status r = run_sweeps(c, nullptr, &st, fused ? c->w2 : nullptr, fused && last);
         if (r != MFC_OK) return r;
-        std::swap(c->w, c->w2);
+        if (fused) std::swap(c->w, c->w2);
+        if (c->six) return run_prims(c, st.qout, last, true);
         return MFC_OK;
     };
-    auto between = [&](const double* q) -> mfc_status { return fused ? MFC_OK : run_prims(c, q, false); };
+    auto between = [&](const double* q) -> mfc_status {
+        return fused || c->six ? MFC_OK : run_prims(c, q, false);
+    };
     if (c->rk_order == 1) {
         // forward Euler, in place: q = q + dt R(q)
         RkStage st{c->q, c->q, c->q, 0.0, 1.0, dt};
@@ -751,8 +764,8 @@ mfc_status mfc_step(mfc_ctx* c, double dt) {
         RkStage st3{c->q, c->q1, c->q, 1.0 / 3.0, 2.0 / 3.0, dt};
         if ((s = stage(st3, true)) != MFC_OK) return s;
     }
-    c->w_valid = fused;
-    c->rate_valid = fused;
+    c->w_valid = fused || c->six;
+    c->rate_valid = fused || c->six;
     return MFC_OK;
 }
 

@@ -1,6 +1,5 @@
-// Finishing a cell (Sec. 3.1, 3.3, 3.4, 2.1, 2.3): characteristic boundary
-// rates, the Kapila coefficients, the six-equation pressure relaxation, and
-// finish_cell (flux difference, sources, RK stage update).
+// Finishing a cell (Sec. 3.1, 3.3, 3.4, 2.1): characteristic boundary
+// rates, the Kapila coefficients, and finish_cell (flux difference, sources, RK stage update).
 #pragma once
 #include "mfc_learned.cuh"
 
@@ -150,160 +149,6 @@ __device__ __forceinline__ void kapila_K_df(const SweepArgs& a, const double* w,
     for (int k = 1; k < NF; ++k) D = df_add(D, df_mul(al[k], pe[k]));
 #pragma unroll
     for (int k = 0; k < NF - 1; ++k) K[k] = df_to_double(df_mul(al[k], df_add(df_div(pe[k], D), {-1.f, 0.f})));
-}
-
-// Six-equation model (Sec. 2.3): pressure relaxation of one cell's conserved
-// state q[NQ] with infinite stiffness, in place, after a Runge-Kutta stage
-// (Saurel, Petitpas & Berry 2009; Schmidmayer et al. 2020).  At fixed mass
-// each phase's energy follows de_k = -p dv_k at the final pressure p, which for
-// a stiffened gas gives the relaxed volume fraction
-//     a_k(p) = (g_k - 1)(E_k0 + a_k0 p) / (g_k (p + pinf_k)),  E_k0 = a_k r_k e_k.
-// The phases taking part are those with a_k0 > 0 and p_k0 + pinf_k > 0
-// (E_k0 > a_k0 pinf_k); the others keep a_k0.  The relaxed pressure solves
-// f(p) = sum_{taking part} a_k(p) - (1 - sum_{others} a_k0) = 0; on
-// p > lo = -min pinf (over the phases taking part) f is convex and falls
-// strictly from +inf to below zero, so the root is unique.
-//  1. FP32 Newton from the pressure the mixture law gives for the total energy
-//     with the old fractions (the root itself for a relaxed state): from the
-//     left of the root Newton rises monotonically to it, from the right it
-//     lands left of it unless it would leave the domain, when the step bisects
-//     [lo, p] instead; at most 60 iterations, ending at a relative step of 2^-20;
-//  2. two Newton steps with f in float-float arithmetic (f' in FP32 suffices:
-//     its error only slows the quadratic convergence to a linear one with
-//     factor ~1e-7), which bring p to ~1e-14 relative;
-//  3. one FP64 Newton step, p1 = p0 - f(p0)/f'(p0), and the new fractions
-//     a_k(p1) = a_k(p0) + a_k'(p0)(p1 - p0) (the second-order remainder is
-//     below FP64 rounding): a fraction near 1 must be right to ~1e-16
-//     absolute, since a trace phase's fraction is 1 minus it;
-//  4. in FP64 the pressure of the total energy with the mixture law of the
-//     new fractions and every phase's energy reset to it.
-// On GB300 an FP64 instruction costs the issue time of ~60 FP32 ones; the
-// iteration is the costly part, hence steps 1-2 (see mfc_df.cuh).
-template <int NF, int NDIM>
-__device__ __noinline__ void relax6(const SweepArgs& a, double* q) {
-    using Lay = Layout<NF, NDIM, true>;
-    constexpr int IM = Lay::IM, IE = Lay::IE, IA = Lay::IA, II = Lay::II;
-    double a0[NF], E0[NF];
-    bool in[NF];
-    double asum = 0.0;
-#pragma unroll
-    for (int k = 0; k < NF - 1; ++k) {
-        a0[k] = q[IA + k];
-        asum += a0[k];
-    }
-    a0[NF - 1] = 1.0 - asum;
-    double target = 1.0;
-    float lo = 0.f;
-    bool any = false;
-#pragma unroll
-    for (int k = 0; k < NF; ++k) {
-        E0[k] = q[II + k];
-        in[k] = a0[k] > 0.0 && E0[k] > a0[k] * a.kpinf[k];
-        if (!in[k]) {
-            target -= a0[k];
-            continue;
-        }
-        lo = any ? fmaxf(lo, -a.kpinff[k]) : -a.kpinff[k];
-        any = true;
-    }
-    if (!any) return;   // no phase can relax: left as is (the CFL check flags it)
-    // mixture-law pressure of the total energy (old fractions, then new ones)
-    double r = q[0], m2 = 0.0;
-#pragma unroll
-    for (int k = 1; k < NF; ++k) r += q[k];
-#pragma unroll
-    for (int d = 0; d < NDIM; ++d) m2 = fma(q[IM + d], q[IM + d], m2);
-    const double eint = q[IE] - 0.5 * m2 * rcp_nr(r);
-    auto mixture_p = [&]() {
-        double G = a.e.G_N, P = a.e.P_N;
-#pragma unroll
-        for (int k = 0; k < NF - 1; ++k) {
-            G = fma(q[IA + k], a.e.dG[k], G);
-            P = fma(q[IA + k], a.e.dP[k], P);
-        }
-        return (eint - P) * rcp_nr(G);
-    };
-    // the phases in float-float (integer splits) and FP32
-    df a0d[NF], E0d[NF], pid[NF], c1d[NF];
-    float a0f[NF], E0f[NF], pif[NF], c1f[NF];
-#pragma unroll
-    for (int k = 0; k < NF; ++k) {
-        a0d[k] = df_from_double(a0[k]);
-        E0d[k] = df_from_double(E0[k]);
-        pid[k] = a.kpinfd[k];
-        c1d[k] = a.rc1d[k];
-        a0f[k] = a0d[k].hi;
-        E0f[k] = E0d[k].hi;
-        pif[k] = a.kpinff[k];
-        c1f[k] = c1d[k].hi;
-    }
-    const df targetd = df_from_double(target);
-    // 1. FP32 Newton
-    float p = (float)mixture_p();
-    if (!(p > lo)) p = lo + fmaxf(fabsf(lo), 1.f);
-    float hi = INFINITY;
-    for (int it = 0; it < 60; ++it) {
-        float f = -targetd.hi, fp = 0.f;
-#pragma unroll
-        for (int k = 0; k < NF; ++k) {
-            if (!in[k]) continue;
-            const float t = rcp_approx(p + pif[k]);
-            f = fmaf(c1f[k] * fmaf(a0f[k], p, E0f[k]), t, f);
-            fp = fmaf(c1f[k] * fmaf(a0f[k], pif[k], -E0f[k]), t * t, fp);
-        }
-        if (f > 0.f) lo = p;
-        else hi = p;
-        float pn = p - f * rcp_approx(fp);
-        if (!(pn > lo && pn < hi)) pn = 0.5f * (lo + (hi < INFINITY ? hi : p));
-        const bool done = fabsf(pn - p) <= 0x1p-20f * fabsf(pn) || !(pn > lo && pn < hi);
-        p = pn;
-        if (done) break;
-    }
-    // 2. float-float Newton steps
-    df pd = {p, 0.f};
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-        df f = df_neg(targetd);
-        float fp = 0.f;
-#pragma unroll
-        for (int k = 0; k < NF; ++k) {
-            if (!in[k]) continue;
-            const df num = df_add(E0d[k], df_mul(a0d[k], pd));
-            const df den = df_add(pd, pid[k]);
-            f = df_add(f, df_mul(c1d[k], df_div(num, den)));
-            const float t = rcp_approx(den.hi);
-            fp = fmaf(c1f[k] * fmaf(a0f[k], pif[k], -E0f[k]), t * t, fp);
-        }
-        pd = df_add(pd, {-(f.hi + f.lo) * rcp_approx(fp), 0.f});
-    }
-    // 3. one FP64 Newton step and the fractions at its end (first order)
-    const double p0 = df_to_double(pd);
-    double ak[NF], dak[NF], f64 = -target, fp64 = 0.0;
-#pragma unroll
-    for (int k = 0; k < NF; ++k) {
-        ak[k] = a0[k];
-        dak[k] = 0.0;
-        if (!in[k]) continue;
-        const double pi = a.kpinf[k];
-        const double t = rcp_nr(p0 + pi);
-        ak[k] = a.rc1[k] * fma(a0[k], p0, E0[k]) * t;
-        dak[k] = a.rc1[k] * fma(a0[k], pi, -E0[k]) * t * t;
-        f64 += ak[k];
-        fp64 += dak[k];
-    }
-    const double dp = df_widen(-(float)f64 * rcp_approx((float)fp64));
-    // 4. new fractions, the pressure of the total energy, the phase energies
-    double an = 1.0;
-#pragma unroll
-    for (int k = 0; k < NF - 1; ++k) {
-        if (in[k]) q[IA + k] = fma(dak[k], dp, ak[k]);
-        an -= q[IA + k];
-    }
-    const double pe = mixture_p();
-#pragma unroll
-    for (int k = 0; k < NF - 1; ++k)
-        q[II + k] = q[IA + k] * fma(a.e.G_N + a.e.dG[k], pe, a.e.P_N + a.e.dP[k]);
-    q[II + NF - 1] = an * fma(a.e.G_N, pe, a.e.P_N);
 }
 
 // Normal rate of a characteristic boundary cell (flat index idx, neighbours
@@ -631,8 +476,8 @@ __device__ __forceinline__ void publish_rate(const SweepArgs& a, const RateAcc& 
 // then store, accumulate or apply the RK stage.
 //
 // Six-equation model (SIX): NQ rows; the phase energies lose a_k p div(u)
-// (cell values), and an RK stage update ends with the pressure relaxation
-// (relax6) before it is stored.
+// (cell values).  The pressure relaxation that ends an RK stage runs in the
+// recovery pass after the sweep (relax_prims_kernel).
 //
 // stg (y/z stream kernels, or null): this lane's operands staged by
 // stage_finish_operands, complete (cp_async_wait_all) before the call.
@@ -740,13 +585,9 @@ __device__ __forceinline__ double finish_cell_rates(const SweepArgs& a, long lon
             }
             if (a.c0 != 0.0) o = fma(a.c0, q0v(v), o);
             qn[v] = o;
-            if constexpr (!SIX) a.qout[v * nc + idx] = o;
+            a.qout[v * nc + idx] = o;
         }
-        if constexpr (SIX) {
-            relax6<NF, NDIM>(a, qn);
-#pragma unroll
-            for (int v = 0; v < NQ; ++v) a.qout[v * nc + idx] = qn[v];
-        } else if constexpr (sizeof(Real) == 8) {
+        if constexpr (sizeof(Real) == 8 && !SIX) {
             // FP64 form only: in the FP32 forms' z sweep (memory-bound, 64
             // registers) the fused recovery spilled and cost more than the
             // separate pass it replaced (mixed 6.27 -> 6.52 ms per step at 256^3)

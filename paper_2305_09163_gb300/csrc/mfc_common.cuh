@@ -107,8 +107,7 @@ struct SweepArgs {
     const void* cbc_rates;  // their cells' normal rates (cbc_rates_kernel), Real, or null
     long long cbc_off[3][2];    // start of direction d, side s in cbc_rates (-1: not characteristic)
     int kapila;             // 1: Kapila model, K div(u) in the volume-fraction rows
-    double kgam[3], kpinf[3];   // Kapila, six-equation model: gamma_k and pi_inf_k of every fluid
-    double rc1[3];              // six-equation relaxation: (gamma_k - 1)/gamma_k
+    double kgam[3], kpinf[3];   // Kapila: gamma_k and pi_inf_k of every fluid
     float kgamf[3], kpinff[3];
     EosConstF ef;           // FP32 kernels: e, eps * 3/4 and g.inv_dx in FP32
     float eps34f;
@@ -116,7 +115,7 @@ struct SweepArgs {
     float inv_dxf[3];
     EosDf ed;               // FP64 kernels: e, eps * 3/4, eps and g.inv_dx in float-float
     df eps34d, epsd, inv_dxd[3];
-    df kgamd[3], kpinfd[3], rc1d[3];   // kgam, kpinf, rc1 in float-float
+    df kgamd[3], kpinfd[3];     // kgam, kpinf in float-float
 };
 
 // Fill the FP32 and float-float constants of a from its FP64 ones (host, after
@@ -157,7 +156,6 @@ inline void sweep_set_constants(SweepArgs& a) {
     for (int k = 0; k < 3; ++k) {
         a.kgamd[k] = df_split(a.kgam[k]);
         a.kpinfd[k] = df_split(a.kpinf[k]);
-        a.rc1d[k] = df_split(a.rc1[k]);
     }
 }
 
@@ -170,6 +168,14 @@ struct PrimArgs {
     int* bad;               // optional: count of non-physical cells
     const float* grid[3];   // non-uniform directions: WENO5 table (GridCol layout), else null
     int grid_stride[3];
+};
+
+// Six-equation model: constants of the pressure relaxation, per phase, in FP64,
+// float-float and FP32 (host: make_relax_const).
+struct RelaxConst {
+    double pinf[3], c1[3], G[3], P[3];   // pi_inf, (gamma - 1)/gamma, 1/(gamma - 1), gamma pi_inf/(gamma - 1)
+    df pinfd[3], c1d[3], P_N, dP[2];     // P_N, dP: as in EosConst
+    float pinff[3], c1f[3], G_N, dG[2];
 };
 
 // Non-uniform grid table of one direction: 28 values per cell (mfc_grid.cu),

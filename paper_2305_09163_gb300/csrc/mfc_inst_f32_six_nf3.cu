@@ -4,4 +4,5 @@
 namespace mfc {
 template cudaError_t launch_sweep<float, 3, false, 5, false, true>(SweepArgs, int, int, cudaStream_t);
 template cudaError_t launch_prims<float, 3, true>(const PrimArgs&, int, bool, cudaStream_t);
+template cudaError_t launch_relax_prims<float, 3>(const PrimArgs&, const RelaxConst&, int, bool, cudaStream_t);
 }  // namespace mfc

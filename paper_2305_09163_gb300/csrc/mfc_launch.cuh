@@ -191,6 +191,22 @@ cudaError_t launch_prims(const PrimArgs& a, int ndim, bool rate, cudaStream_t s)
     return cudaGetLastError();
 }
 
+// Six-equation model: relaxation and primitive recovery of a stage's new state.
+template <typename Real, int NF>
+cudaError_t launch_relax_prims(const PrimArgs& a, const RelaxConst& c, int ndim, bool rate, cudaStream_t s) {
+    const unsigned blocks = elem_blocks(a.g.ncell);
+    switch (ndim * 2 + (rate ? 1 : 0)) {
+        case 2: relax_prims_kernel<Real, NF, 1, false><<<blocks, kElemThreads, 0, s>>>(a, c); break;
+        case 3: relax_prims_kernel<Real, NF, 1, true><<<blocks, kElemThreads, 0, s>>>(a, c); break;
+        case 4: relax_prims_kernel<Real, NF, 2, false><<<blocks, kElemThreads, 0, s>>>(a, c); break;
+        case 5: relax_prims_kernel<Real, NF, 2, true><<<blocks, kElemThreads, 0, s>>>(a, c); break;
+        case 6: relax_prims_kernel<Real, NF, 3, false><<<blocks, kElemThreads, 0, s>>>(a, c); break;
+        case 7: relax_prims_kernel<Real, NF, 3, true><<<blocks, kElemThreads, 0, s>>>(a, c); break;
+        default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
 // Characteristic boundary rates (cbc_rates_kernel): total = boundary cells.
 template <typename Real, int NF>
 cudaError_t launch_cbc(const SweepArgs& a, int ndim, long long total, cudaStream_t s) {
@@ -254,6 +270,28 @@ inline EosConst make_eos_const(int N, const double* gamma, const double* pi_inf)
         e.dB[k] = on ? gamma[k] * pi_inf[k] - gamma[N - 1] * pi_inf[N - 1] : 0.0;
     }
     return e;
+}
+
+// Host: the six-equation relaxation's constants in the precisions it takes.
+inline RelaxConst make_relax_const(int N, const double* gamma, const double* pi_inf, const EosConst& e) {
+    RelaxConst c{};
+    for (int k = 0; k < N; ++k) {
+        c.pinf[k] = pi_inf[k];
+        c.c1[k] = (gamma[k] - 1.0) / gamma[k];
+        c.G[k] = k < N - 1 ? e.G_N + e.dG[k] : e.G_N;
+        c.P[k] = k < N - 1 ? e.P_N + e.dP[k] : e.P_N;
+        c.pinfd[k] = df_split(c.pinf[k]);
+        c.c1d[k] = df_split(c.c1[k]);
+        c.pinff[k] = (float)c.pinf[k];
+        c.c1f[k] = c.c1d[k].hi;
+    }
+    c.P_N = df_split(e.P_N);
+    c.G_N = (float)e.G_N;
+    for (int k = 0; k < 2; ++k) {
+        c.dP[k] = df_split(e.dP[k]);
+        c.dG[k] = (float)e.dG[k];
+    }
+    return c;
 }
 
 // Host: cells per thread along direction dir of a marching sweep; halved while
@@ -344,6 +382,10 @@ extern template cudaError_t launch_prims<double, 2, true>(const PrimArgs&, int, 
 extern template cudaError_t launch_prims<double, 3, true>(const PrimArgs&, int, bool, cudaStream_t);
 extern template cudaError_t launch_prims<float, 2, true>(const PrimArgs&, int, bool, cudaStream_t);
 extern template cudaError_t launch_prims<float, 3, true>(const PrimArgs&, int, bool, cudaStream_t);
+extern template cudaError_t launch_relax_prims<double, 2>(const PrimArgs&, const RelaxConst&, int, bool, cudaStream_t);
+extern template cudaError_t launch_relax_prims<double, 3>(const PrimArgs&, const RelaxConst&, int, bool, cudaStream_t);
+extern template cudaError_t launch_relax_prims<float, 2>(const PrimArgs&, const RelaxConst&, int, bool, cudaStream_t);
+extern template cudaError_t launch_relax_prims<float, 3>(const PrimArgs&, const RelaxConst&, int, bool, cudaStream_t);
 extern template cudaError_t launch_cons6<2>(const Geometry&, const EosConst&, const double*, double*, int, cudaStream_t);
 extern template cudaError_t launch_cons6<3>(const Geometry&, const EosConst&, const double*, double*, int, cudaStream_t);
 extern template cudaError_t launch_cons<1>(const Geometry&, const EosConst&, const double*, double*, int, cudaStream_t);
