@@ -32,6 +32,8 @@
 
 using namespace mfc;
 
+cudaError_t mfc_launch_mlp_reduce(const float* work, int parts, float* grad, float* loss, cudaStream_t s);
+
 namespace {
 
 constexpr int kTile = 128;                  // samples per tile (MMA M)
@@ -386,17 +388,6 @@ __global__ void __launch_bounds__(kTile) mlp_grad_tc_kernel(const float* __restr
     if (warp == 0) tc::tmem_dealloc(tm, 256);
 }
 
-// Deterministic sum of the per-CTA partials, one thread per slot.
-__global__ void mlp_tc_reduce_kernel(const float* __restrict__ work, int parts, float* __restrict__ grad,
-                                     float* __restrict__ loss) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p > kMlpParams) return;
-    float s = 0.f;
-    for (int w = 0; w < parts; ++w) s += work[(long long)w * kTcStride + p];
-    if (p < kMlpParams) grad[p] = s;
-    else if (loss) *loss = s;
-}
-
 unsigned grid_for(long long B, int per_sm) {
     long long tiles = (B + kTile - 1) / kTile;
     const long long cap = 152LL * per_sm;
@@ -430,8 +421,7 @@ mfc_status mfc_mlp_grad(const float* params, const float* x, const float* phat, 
     static_assert(2LL * 152 * kTcStride <= MFC_MLP_WORK_FLOATS, "workspace holds every CTA's partial");
     mlp_grad_tc_kernel<<<blocks, kTile, kGradSmem, s>>>(params, x, phat, target, mask, batch, lam, work);
     if (cudaGetLastError() != cudaSuccess) return MFC_ERR_CUDA;
-    mlp_tc_reduce_kernel<<<(kTcStride + 127) / 128, 128, 0, s>>>(work, (int)blocks, grad, loss);
-    return cudaGetLastError() == cudaSuccess ? MFC_OK : MFC_ERR_CUDA;
+    return mfc_launch_mlp_reduce(work, (int)blocks, grad, loss, s) == cudaSuccess ? MFC_OK : MFC_ERR_CUDA;
 }
 
 int mfc_mlp_tc_status(void) {
