@@ -413,137 +413,299 @@ __device__ double weno5_js(const double* v, double eps) {
     return (a0 * p0 + a1 * p1 + a2 * p2) / (a0 + a1 + a2);
 }
 
-__global__ void harvest_kernel(const double* __restrict__ wf, int nxf, int nyf, int nzf, int ndim, int ns,
-                               double eps, double tau, long long nsamp, unsigned long long seed,
-                               float* __restrict__ xo, float* __restrict__ po, float* __restrict__ to,
-                               float* __restrict__ so, float* __restrict__ jo) {
-    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= nsamp) return;
-    const long long nf = (long long)nxf * nyf * nzf;
-    const int nfd[3] = {nxf, nyf, nzf};
-    int nc[3];
-    for (int a = 0; a < 3; ++a) nc[a] = a < ndim ? nfd[a] / 2 : 1;
-    const unsigned long long h0 = mix64(seed ^ mix64((unsigned long long)k));
-    const unsigned long long h1 = mix64(h0), h2 = mix64(h1), h3 = mix64(h2);
-    const int d = (int)(h0 % (unsigned long long)ndim);
-    const int side = (int)((h0 >> 20) & 1ULL);
-    const int var = (int)((h0 >> 24) % (unsigned long long)ns);
-    const int I = 2 + (int)(h1 % (unsigned long long)(nc[d] - 6));
-    int cc[3];
-    cc[0] = (int)(h2 % (unsigned long long)nc[0]);
-    cc[1] = (int)((h2 >> 21) % (unsigned long long)nc[1]);
-    cc[2] = (int)((h3) % (unsigned long long)nc[2]);
-    const long long sf[3] = {1, (long long)nxf, (long long)nxf * nyf};
-    const double* wv = wf + (long long)var * nf;
-    const int nchild = 1 << ndim;
-    // coarse values of cells I-2..I+3 along d
-    double W[6];
-    for (int m = 0; m < 6; ++m) {
-        int c[3] = {cc[0], cc[1], cc[2]};
-        c[d] = I - 2 + m;
-        double s = 0.0;
-        for (int ch = 0; ch < nchild; ++ch) {
-            long long idx = 0;
-            for (int a = 0; a < 3; ++a) {
-                const int f = a < ndim ? 2 * c[a] + ((ch >> a) & 1) : 0;
-                idx += f * sf[a];
-            }
-            s += wv[idx];
-        }
-        W[m] = s / nchild;
+// WENO5-JS increments at the right edge of the middle cell of two stencils side
+// by side, X_k the four differences of each (weno5_increments_pair with a stencil
+// of its own in every lane), in float-float; optionally the smoothness
+// indicators without their 4/3 factor.  e = 3/4 eps.
+__device__ __forceinline__ df2 weno5_right_pair(df2 X0, df2 X1, df2 X2, df2 X3, df2 e, df2* beta = nullptr) {
+    const df2 S1 = df2_mul(X1, X1), S2 = df2_mul(X2, X2);
+    const df2 b0 = df2_add_fast(df2_add_fast(df2_mul(X0, X0), df2_mul_f(df2_mul(X1, X0), f2(-2.75f))),
+                                df2_mul_f(S1, f2(2.5f)));
+    const df2 b1 = df2_add_fast(df2_add_fast(S1, S2), df2_mul_f(df2_mul(X1, X2), f2(-1.25f)));
+    const df2 b2 = df2_add_fast(df2_add_fast(df2_mul(X3, X3), df2_mul_f(df2_mul(X2, X3), f2(-2.75f))),
+                                df2_mul_f(S2, f2(2.5f)));
+    if (beta) {
+        beta[0] = b0;
+        beta[1] = b1;
+        beta[2] = b2;
     }
-    double st[5];
-    for (int m = 0; m < 5; ++m) st[m] = side == 0 ? W[m] : W[5 - m];
-    // fine target: faces between fine cells 2I+1 and 2I+2 along d
+    const df2 T0 = df2_add_fast(e, b0), T1 = df2_add_fast(e, b1), T2 = df2_add_fast(e, b2);
+    const float2 m = make_float2(fminf(T0.hi.x, fminf(T1.hi.x, T2.hi.x)), fminf(T0.hi.y, fminf(T1.hi.y, T2.hi.y)));
+    const df2 g0 = df2_div_f(m, T0), g1 = df2_div_f(m, T1), g2 = df2_div_f(m, T2);
+    const df2 w0 = df2_mul(g0, g0), w1 = df2_mul_f(df2_mul(g1, g1), f2(6.f)), w2 = df2_mul_f(df2_mul(g2, g2), f2(3.f));
+    const df2 P0 = df2_add_fast(df2_mul_f(X1, f2(5.f)), df2_mul_pow2(X0, f2(-2.f)));
+    const df2 P1 = df2_add_fast(X1, df2_mul_pow2(X2, f2(2.f)));
+    const df2 P2 = df2_add_fast(df2_mul_pow2(X2, f2(4.f)), df2_neg(X3));
+    const df2 num = df2_add_fast(df2_add_fast(df2_mul(w0, P0), df2_mul(w1, P1)), df2_mul(w2, P2));
+    return df2_div(num, df2_mul_f(df2_add_fast(df2_add_fast(w0, w1), w2), f2(6.f)));
+}
+
+// One sample's outputs in plain FP64, for values outside the range of the
+// float-float form below: differences of 1e18 and more or of less than 2^-60 of
+// them all, non-finite values, eps outside [1e-30, 1].  f6: per fine face the six
+// values across it.
+__device__ __noinline__ void harvest_sample_f64(const double* st, const double* f6, int ntr, double eps, double tau,
+                                                float* x, float* ph, float* to, float* so, float* jo) {
     double tgt = 0.0;
-    const int ntr = nchild / 2;
     for (int ch = 0; ch < ntr; ++ch) {
-        long long base = 0;
-        int bit = 0;
-        for (int a = 0; a < 3; ++a) {
-            if (a == d) continue;
-            const int f = a < ndim ? 2 * cc[a] + ((ch >> bit) & 1) : 0;
-            if (a < ndim) ++bit;
-            base += f * sf[a];
-        }
-        double f6[6];
-        for (int m = 0; m < 6; ++m) f6[m] = wv[base + (long long)(2 * I - 1 + m) * sf[d]];
-        const double l = weno5_js(f6, eps);
-        const double rv[5] = {f6[5], f6[4], f6[3], f6[2], f6[1]};
-        const double r = weno5_js(rv, eps);
-        tgt += 0.5 * (l + r);
+        const double* f = f6 + 6 * ch;
+        const double l = weno5_js(f, eps);
+        const double rv[5] = {f[5], f[4], f[3], f[2], f[1]};
+        tgt += 0.5 * (l + weno5_js(rv, eps));
     }
     tgt /= ntr;
     const double c = st[2];
     double s = 0.0;
     for (int m = 0; m < 5; ++m) s = fmax(s, fabs(st[m] - c));
     const double tn = (tgt - c) / (s + 1e-30);
-    // A stencil flat to FP32 resolution of its centre value carries no shape to
-    // learn (its normalised target would be round-off); such samples, and any
-    // whose fine target lies far outside the stencil's range, are stored as
-    // zeros with smooth = 0 so they add nothing to the loss.
-    if (!(s > 1e-7 * fabs(c)) || !(s > 1e-300) || !(fabs(tn) <= 8.0)) {
-        for (int m = 0; m < 5; ++m) xo[k * 5 + m] = 0.f;
-        po[k * 3 + 0] = po[k * 3 + 1] = po[k * 3 + 2] = 0.f;
-        to[k] = 0.f;
-        jo[k] = 0.f;
-        so[k] = 0.f;
-        return;
-    }
+    for (int m = 0; m < 5; ++m) x[m] = 0.f;
+    ph[0] = ph[1] = ph[2] = *to = *jo = *so = 0.f;
+    if (!(s > 1e-7 * fabs(c)) || !(s > 1e-300) || !(fabs(tn) <= 8.0)) return;
     s += 1e-30;
-    for (int m = 0; m < 5; ++m) xo[k * 5 + m] = (float)((st[m] - c) / s);
+    for (int m = 0; m < 5; ++m) x[m] = (float)((st[m] - c) / s);
     const double p0 = (2.0 * st[0] - 7.0 * st[1] + 11.0 * st[2]) / 6.0;
     const double p1 = (-st[1] + 5.0 * st[2] + 2.0 * st[3]) / 6.0;
     const double p2 = (2.0 * st[2] + 5.0 * st[3] - st[4]) / 6.0;
-    po[k * 3 + 0] = (float)((p0 - c) / s);
-    po[k * 3 + 1] = (float)((p1 - c) / s);
-    po[k * 3 + 2] = (float)((p2 - c) / s);
-    to[k] = (float)tn;
-    jo[k] = (float)((weno5_js(st, eps) - c) / s);
+    ph[0] = (float)((p0 - c) / s);
+    ph[1] = (float)((p1 - c) / s);
+    ph[2] = (float)((p2 - c) / s);
+    *to = (float)tn;
+    *jo = (float)((weno5_js(st, eps) - c) / s);
     // discontinuity sensor (the same test the learned sweep applies)
     const double D0 = st[1] - st[0], D1 = st[2] - st[1], D2 = st[3] - st[2], D3 = st[4] - st[3];
     const double bb0 = 2.5 * D1 * D1 - 2.75 * D1 * D0 + D0 * D0;
     const double bb1 = D1 * D1 + D2 * D2 - 1.25 * D1 * D2;
     const double bb2 = 2.5 * D2 * D2 - 2.75 * D2 * D3 + D3 * D3;
     const double bmax = fmax(bb0, fmax(bb1, bb2)), bmin = fmin(bb0, fmin(bb1, bb2));
-    so[k] = bmax > tau * (bmin + 1e-6 * s * s) ? 0.f : 1.f;
+    *so = bmax > tau * (bmin + 1e-6 * s * s) ? 0.f : 1.f;
 }
 
-__global__ void __launch_bounds__(256) prims_out_kernel(const double* __restrict__ q, double* __restrict__ w,
-                                                        long long nc, int nf, int ndim, EosConst e, int six) {
-    // generic (runtime NF, NDIM) FP64 primitive recovery for output; the
-    // six-equation model (six) appends the phase pressures
-    // p_k = (a_k r_k e_k / a_k - P_k)/G_k
-    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int ns = 2 * nf + ndim, IM = nf, IE = nf + ndim, IA = nf + ndim + 1;
-        double rho = 0.0;
-        for (int k2 = 0; k2 < nf; ++k2) rho += q[k2 * nc + i];
-        double G = e.G_N, Pm = e.P_N;
-        for (int k2 = 0; k2 < nf - 1; ++k2) {
-            G = fma(q[(IA + k2) * nc + i], e.dG[k2], G);
-            Pm = fma(q[(IA + k2) * nc + i], e.dP[k2], Pm);
-        }
-        double ke = 0.0;
-        for (int a = 0; a < ndim; ++a) {
-            const double u = q[(IM + a) * nc + i] / rho;
-            w[(IM + a) * nc + i] = u;
-            ke = fma(q[(IM + a) * nc + i], u, ke);
-        }
-        for (int k2 = 0; k2 < nf; ++k2) w[k2 * nc + i] = q[k2 * nc + i];
-        w[IE * nc + i] = (q[IE * nc + i] - 0.5 * ke - Pm) / G;
-        for (int k2 = IA; k2 < ns; ++k2) w[k2 * nc + i] = q[k2 * nc + i];
-        if (six) {
-            double aN = 1.0;
-            for (int k2 = 0; k2 < nf; ++k2) {
-                const double ak = k2 < nf - 1 ? q[(IA + k2) * nc + i] : aN;
-                if (k2 < nf - 1) aN -= ak;
-                const double Gk = k2 < nf - 1 ? e.G_N + e.dG[k2] : e.G_N;
-                const double Pk = k2 < nf - 1 ? e.P_N + e.dP[k2] : e.P_N;
-                w[(ns + k2) * nc + i] = (q[(ns + k2) * nc + i] / ak - Pk) / Gk;
+__device__ __forceinline__ unsigned abs_hi(double d) { return (unsigned)__double2hiint(d) & 0x7FFFFFFFu; }
+
+// A stencil flat to FP32 resolution of its centre value carries no shape to
+// learn (its normalised target would be round-off); such samples, and any
+// whose fine target lies far outside the stencil's range, are stored as
+// zeros with smooth = 0 so they add nothing to the loss.
+//
+// In plain FP64 (nine WENO5-JS values, ~80 divisions) a sample took ~1,400 FP64
+// instructions and the kernel was bound by them: 500,000 samples of a 160^3
+// field 1.10 ms, now 0.22 ms, bound by the gather (72 values of 8 bytes per
+// sample from as many sectors, 0.79 GB from DRAM).  Here FP64 forms the coarse means and all differences; weights,
+// increments and normalised values are float-float (mfc_df.cuh, ~2^-46 of the
+// differences, far below the FP32 they are stored in), the two sides of a fine
+// face in the lanes of packed instructions.  Everything is taken relative to the
+// centre value, so nothing cancels where the stencil is small against it.
+template <int NDIM>
+__global__ void __launch_bounds__(128) harvest_kernel(const double* __restrict__ wf, int nxf, int nyf, int nzf, int ns,
+                                                      double eps, double tau, df eps34, df taud, df scale,
+                                                      bool eps_in_range,
+                                                      long long nsamp, unsigned long long seed,
+                                                      float* __restrict__ xo, float* __restrict__ po,
+                                                      float* __restrict__ to, float* __restrict__ so,
+                                                      float* __restrict__ jo) {
+    const long long k = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (k >= nsamp) return;
+    const long long nf = (long long)nxf * nyf * nzf;
+    const int nc[3] = {nxf / 2, NDIM > 1 ? nyf / 2 : 1, NDIM > 2 ? nzf / 2 : 1};
+    const unsigned long long h0 = mix64(seed ^ mix64((unsigned long long)k));
+    const unsigned long long h1 = mix64(h0), h2 = mix64(h1), h3 = mix64(h2);
+    const int d = (int)(h0 % (unsigned long long)NDIM);
+    const int side = (int)((h0 >> 20) & 1ULL);
+    const int var = (int)((h0 >> 24) % (unsigned long long)ns);
+    const int nd = d == 0 ? nc[0] : d == 1 ? nc[1] : nc[2];
+    const int I = 2 + (int)(h1 % (unsigned long long)(nd - 6));
+    const int cc[3] = {(int)(h2 % (unsigned long long)nc[0]), (int)((h2 >> 21) % (unsigned long long)nc[1]),
+                       (int)(h3 % (unsigned long long)nc[2])};
+    const long long sf[3] = {1, (long long)nxf, (long long)nxf * nyf};
+    const long long sd = d == 0 ? sf[0] : d == 1 ? sf[1] : sf[2];
+    // first fine cell of the coarse column: transverse coordinates 2 cc, 0 along d
+    long long base = (long long)var * nf;
+#pragma unroll
+    for (int a = 0; a < NDIM; ++a) base += a == d ? 0 : 2 * cc[a] * sf[a];
+    // strides of the transverse directions, in their order
+    const long long t1 = d == 0 ? sf[1] : sf[0], t2 = d == 2 ? sf[1] : sf[2];
+    constexpr int NTR = 1 << (NDIM - 1);
+    const double* col = wf + base + (long long)(2 * (I - 2)) * sd;   // fine cells 2I-4 .. 2I+7 along d
+    // coarse values of cells I-2..I+3 along d: mean of the 2^d children, summed in
+    // the children's order (x fastest); the fine values across the face are among them
+    double W[6], f6[NTR][6];
+#pragma unroll
+    for (int m = 0; m < 6; ++m) {
+        double v[2][NTR];
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+            for (int t = 0; t < NTR; ++t) {
+                v[h][t] = __ldg(col + (2 * m + h) * sd + (t & 1 ? t1 : 0) + (t & 2 ? t2 : 0));
+                const int j = 2 * m + h - 3;   // f6 holds fine cells 2I-1 .. 2I+4
+                if (j >= 0 && j < 6) f6[t][j] = v[h][t];
             }
+        double s = 0.0;
+#pragma unroll
+        for (int ch = 0; ch < 2 * NTR; ++ch) {
+            // child ch: bit a = fine offset in direction a
+            double u0 = v[ch & 1][(ch >> 1) & (NTR - 1)];                                    // d == 0
+            if constexpr (NDIM > 1) {
+                const double u1 = v[(ch >> 1) & 1][(ch & 1) | ((ch >> 1) & (NTR - 2))];      // d == 1
+                u0 = d == 0 ? u0 : u1;
+            }
+            if constexpr (NDIM > 2) {
+                const double u2 = v[(ch >> 2) & 1][ch & 3];                                  // d == 2
+                u0 = d == 2 ? u2 : u0;
+            }
+            s += u0;
+        }
+        W[m] = s * (1.0 / (2 * NTR));
+    }
+    double st[5];
+#pragma unroll
+    for (int m = 0; m < 5; ++m) st[m] = side == 0 ? W[m] : W[5 - m];
+    const double c = st[2];
+    float x[5] = {0.f, 0.f, 0.f, 0.f, 0.f}, ph[3] = {0.f, 0.f, 0.f}, tv = 0.f, sv = 0.f, jv = 0.f;
+    // the stencil about its centre; s its largest distance from it (bit patterns
+    // of non-negative doubles order as integers)
+    double dm[5];
+    unsigned long long sb = 0;
+    unsigned big = abs_hi(c);
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+        dm[m] = st[m] - c;
+        const unsigned long long u = (unsigned long long)__double_as_longlong(dm[m]) & 0x7FFFFFFFFFFFFFFFULL;
+        sb = u > sb ? u : sb;
+    }
+    const double s = __longlong_as_double((long long)sb);
+    double e[NTR][5];
+#pragma unroll
+    for (int t = 0; t < NTR; ++t)
+#pragma unroll
+        for (int j = 0; j < 5; ++j) {
+            e[t][j] = f6[t][j + 1] - f6[t][j];
+            big = max(big, abs_hi(e[t][j]));
+        }
+    big = max(big, (unsigned)(sb >> 32));
+    constexpr unsigned kMax = (1023u + 59u) << 20, kMin = (1023u - 60u) << 20;   // 5.8e17, 8.7e-19
+    const bool flat = !(s > 1e-7 * fabs(c)) || !(s > 1e-300);
+    if (!eps_in_range || big >= kMax || (!flat && (unsigned)(sb >> 32) < kMin)) {
+        harvest_sample_f64(st, &f6[0][0], NTR, eps, tau, x, ph, &tv, &sv, &jv);
+    } else if (!flat) {
+        const df2 ep = df2_make(eps34, eps34);
+        // fine target about c: mean over the fine faces of both sides' edge values
+        df inc = {0.f, 0.f};
+        double mid = 0.0;
+#pragma unroll
+        for (int t = 0; t < NTR; ++t) {
+            df E[5];
+#pragma unroll
+            for (int j = 0; j < 5; ++j) E[j] = df_from_double(e[t][j]);
+            const df2 r = weno5_right_pair(df2_make(E[0], df_neg(E[4])), df2_make(E[1], df_neg(E[3])),
+                                           df2_make(E[2], df_neg(E[2])), df2_make(E[3], df_neg(E[1])), ep);
+            inc = df_add(inc, df_add(df2_x(r), df2_y(r)));
+            mid += (f6[t][2] - c) + (f6[t][3] - c);
+        }
+        const double tgt = (mid + df_to_double(inc)) * (0.5 / NTR);
+        const df S = df_from_double(s + 1e-30);
+        const df tn = df_div(df_from_double(tgt), S);
+        if (fabsf(tn.hi) <= 8.f && !(fabsf(tn.hi) == 8.f && (tn.hi > 0.f ? tn.lo > 0.f : tn.lo < 0.f))) {
+            df dd[5], beta[3];
+#pragma unroll
+            for (int m = 0; m < 5; ++m) {
+                dd[m] = df_from_double(dm[m]);
+                x[m] = m == 2 ? 0.f : df_div(dd[m], S).hi;
+            }
+            df X[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) X[j] = df_from_double(st[j + 1] - st[j]);
+            df2 b2[3];
+            const df2 r = weno5_right_pair(df2_make(X[0], X[0]), df2_make(X[1], X[1]), df2_make(X[2], X[2]),
+                                           df2_make(X[3], X[3]), ep, b2);
+            jv = df_div(df2_x(r), S).hi;
+            const df S6 = df_mul_f(S, 6.f);
+            ph[0] = df_div(df_add(df_mul_pow2(dd[0], 2.f), df_mul_f(dd[1], -7.f)), S6).hi;
+            ph[1] = df_div(df_add(df_mul_pow2(dd[3], 2.f), df_neg(dd[1])), S6).hi;
+            ph[2] = df_div(df_add(df_mul_f(dd[3], 5.f), df_neg(dd[4])), S6).hi;
+            tv = tn.hi;
+            // discontinuity sensor (the same test the learned sweep applies)
+#pragma unroll
+            for (int q = 0; q < 3; ++q) beta[q] = df2_x(b2[q]);
+            const df bmax = df_max(beta[0], df_max(beta[1], beta[2])), bmin = df_min(beta[0], df_min(beta[1], beta[2]));
+            const df lim = df_mul(taud, df_add(bmin, df_mul(df_mul(S, S), scale)));
+            sv = df_lt(lim, bmax) ? 0.f : 1.f;
         }
     }
+#pragma unroll
+    for (int m = 0; m < 5; ++m) xo[k * 5 + m] = x[m];
+#pragma unroll
+    for (int m = 0; m < 3; ++m) po[k * 3 + m] = ph[m];
+    to[k] = tv;
+    so[k] = sv;
+    jo[k] = jv;
+}
+
+// n / d from the FP64 Newton reciprocal r of d, finished with the exact residual
+// (Markstein): the rounding of a division; anything not finite is divided (out of
+// line: inlined, the division ran speculatively in every lane, 58 FP64
+// instructions per cell instead of 27).
+__device__ __noinline__ double div_slow(double n, double d) { return n / d; }
+__device__ __forceinline__ double div_by(double n, double d, double r) {
+    const double q = n * r;
+    const double res = fma(fma(-q, d, n), r, q);
+    return abs_hi(res) < 0x7FF00000u ? res : div_slow(n, d);
+}
+
+// FP64 primitive recovery for output; the six-equation model (SIX) appends the
+// phase pressures p_k = (a_k r_k e_k / a_k - P_k)/G_k.  One template per model, so
+// that rows are addressed at compile time and a cell's loads go out together, and
+// two reciprocals for the d + 1 divisions; the kernel is bound by FP64
+// instructions (26 per cell, the FP64 pipe 90% busy).  160^3, two fluids: 312 us
+// with run-time loops and divisions, 193 us now.
+template <int NF, int NDIM, bool SIX>
+__global__ void __launch_bounds__(256) prims_out_kernel(const double* __restrict__ q, double* __restrict__ w,
+                                                        long long nc, EosConst e) {
+    using Lay = Layout<NF, NDIM, SIX>;
+    constexpr int NS = Lay::NS, NQ = Lay::NQ, IM = Lay::IM, IE = Lay::IE, IA = Lay::IA;
+    for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc;
+         i += (long long)gridDim.x * blockDim.x) {
+        double s[NQ];
+#pragma unroll
+        for (int v = 0; v < NQ; ++v) s[v] = __ldg(q + v * nc + i);
+        double rho = s[0], G = e.G_N, P = e.P_N, ke = 0.0;
+#pragma unroll
+        for (int k = 1; k < NF; ++k) rho += s[k];
+#pragma unroll
+        for (int k = 0; k < NF - 1; ++k) {
+            G = fma(s[IA + k], e.dG[k], G);
+            P = fma(s[IA + k], e.dP[k], P);
+        }
+        const double irho = rcp_nr(rho);
+#pragma unroll
+        for (int d = 0; d < NDIM; ++d) {
+            const double u = div_by(s[IM + d], rho, irho);
+            ke = fma(s[IM + d], u, ke);
+            s[IM + d] = u;
+        }
+        s[IE] = div_by(s[IE] - 0.5 * ke - P, G, rcp_nr(G));
+        if constexpr (SIX) {
+            double aN = 1.0;
+#pragma unroll
+            for (int k = 0; k < NF; ++k) {
+                const double ak = k < NF - 1 ? s[IA + k] : aN;
+                if (k < NF - 1) aN -= ak;
+                const double Gk = k < NF - 1 ? e.G_N + e.dG[k] : e.G_N;
+                const double Pk = k < NF - 1 ? e.P_N + e.dP[k] : e.P_N;
+                s[NS + k] = (s[NS + k] / ak - Pk) / Gk;
+            }
+        }
+#pragma unroll
+        for (int v = 0; v < NQ; ++v) w[v * nc + i] = s[v];
+    }
+}
+
+template <int NF, bool SIX>
+void launch_prims_out(const double* q, double* w, long long nc, int ndim, const EosConst& e, unsigned blocks,
+                      cudaStream_t s) {
+    if (ndim == 1) prims_out_kernel<NF, 1, SIX><<<blocks, 256, 0, s>>>(q, w, nc, e);
+    else if (ndim == 2) prims_out_kernel<NF, 2, SIX><<<blocks, 256, 0, s>>>(q, w, nc, e);
+    else prims_out_kernel<NF, 3, SIX><<<blocks, 256, 0, s>>>(q, w, nc, e);
 }
 
 // One warp: the per-lane MMA fragments of a parameter blob, for the sweeps.
@@ -572,7 +734,17 @@ cudaError_t mfc_launch_prims_out(const double* q, double* w, long long nc, int n
                                  int six, cudaStream_t s) {
     long long b = (nc + 255) / 256;
     if (b > 152 * 16) b = 152 * 16;
-    prims_out_kernel<<<(unsigned)b, 256, 0, s>>>(q, w, nc, nf, ndim, e, six);
+    const unsigned blocks = (unsigned)b;
+    if (six) {
+        if (nf == 2) launch_prims_out<2, true>(q, w, nc, ndim, e, blocks, s);
+        else launch_prims_out<3, true>(q, w, nc, ndim, e, blocks, s);
+    } else if (nf == 1) {
+        launch_prims_out<1, false>(q, w, nc, ndim, e, blocks, s);
+    } else if (nf == 2) {
+        launch_prims_out<2, false>(q, w, nc, ndim, e, blocks, s);
+    } else {
+        launch_prims_out<3, false>(q, w, nc, ndim, e, blocks, s);
+    }
     return cudaGetLastError();
 }
 
@@ -623,8 +795,16 @@ mfc_status mfc_harvest(const double* w_fine, int nxf, int nyf, int nzf, int num_
     }
     const int ns = 2 * num_fluids + ndim;
     const long long blocks = (n_samples + 127) / 128;
-    harvest_kernel<<<(unsigned)blocks, 128, 0, static_cast<cudaStream_t>(stream)>>>(
-        w_fine, nxf, nyf, nzf, ndim, ns, weno_eps, tau, n_samples, seed, x, phat, target, smooth, js);
+    const df e34 = df_split(0.75 * weno_eps), taud = df_split(tau), scale = df_split(1e-6);
+    const bool in_range = weno_eps >= 1e-30 && weno_eps <= 1.0 && tau >= 1e-30 && tau <= 1e30;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    auto go = [&](auto kernel) {
+        kernel<<<(unsigned)blocks, 128, 0, st>>>(w_fine, nxf, nyf, nzf, ns, weno_eps, tau, e34, taud, scale, in_range,
+                                                 n_samples, seed, x, phat, target, smooth, js);
+    };
+    if (ndim == 1) go(harvest_kernel<1>);
+    else if (ndim == 2) go(harvest_kernel<2>);
+    else go(harvest_kernel<3>);
     return cudaGetLastError() == cudaSuccess ? MFC_OK : MFC_ERR_CUDA;
 }
 
