@@ -37,33 +37,34 @@ namespace mfc {
 // evaluates the c+1/2 formula on the stencil, lane y the same formula on the
 // mirrored stencil (-D3, -D2, -D1, -D0), which is the edge at c-1/2 (b0 and b2
 // trade places, the candidates above become the eR ones).  b1, its weight and
-// m are common to both edges and are formed once.  Sums use the fast
-// float-float addition: its error, ~2^-44 of the operands, is relative to the
-// stencil's differences, far inside the path's parity tolerance; scalings by
-// powers of two are exact.  (256^3 FP64 step: 39.0 -> 35.9 ms against the same
-// arithmetic in scalar FP32 instructions.)
+// m are common to both edges and are formed once.  Products, sums and quotients
+// leave their results unnormalised (mfc_df.cuh); the weights alone, which are
+// squares of quotients and multiply everything after them, are renormalised
+// (without it the right-hand side's error against 64 bits grew by 7% where the
+// increments dominate).  ~290 instructions per variable and cell; with normalised
+// operations and the three-product indicators ~430 (256^3 x / y sweep 3.40 / 3.42
+// -> 2.91 / 2.78 ms, error unchanged).
+// The indicators are formed as b0 = D0^2 + D1 (5/2 D1 - 11/4 D0), b2 mirrored, and
+// b1 = D1^2 + D2 (D2 - 5/4 D1): two products instead of three.
 __device__ __forceinline__ df2 weno5_increments_pair(const df (&D)[4], df e) {
     const df2 X0 = df2_make(D[0], df_neg(D[3])), X1 = df2_make(D[1], df_neg(D[2]));
     const df2 X2 = df2_swap(df2_neg(X1)), X3 = df2_swap(df2_neg(X0));   // (D2, -D1), (D3, -D0)
-    const df2 SX1 = df2_mul(X1, X1);                                     // (D1^2, D2^2)
-    const df2 B = df2_add_fast(df2_add_fast(df2_mul(X0, X0), df2_mul_f(df2_mul(X1, X0), f2(-2.75f))),
-                               df2_mul_f(SX1, f2(2.5f)));                // (b0, b2)
-    const df b1 = df_add_fast(df_add_fast(df2_x(SX1), df2_y(SX1)), df_mul_f(df_mul(D[1], D[2]), -1.25f));
-    const df2 T = df2_add_fast(df2_make(e, e), B);                       // (t0, t2)
-    const df t1 = df_add_fast(e, b1);
+    const df2 V = df2_sum(df2_scale(X1, f2(2.5f)), df2_scale(X0, f2(-2.75f)));
+    const df2 B = df2_sum(df2_square(X0), df2_prod(X1, V));              // (b0, b2)
+    const df b1 = df_sum(df_square(D[1]), df_prod(D[2], df_sum(D[2], df_scale(D[1], -1.25f))));
+    const df2 T = df2_sum(B, df2_make(e, e));                            // (t0, t2)
+    const df t1 = df_sum(b1, e);
     const float m = fminf(T.hi.x, fminf(t1.hi, T.hi.y));
-    const df2 G = df2_div_f(f2(m), T);                                   // (g0, g2)
-    const df g1 = df_div_f(m, t1);
-    const df2 Q = df2_mul(G, G);                                         // (q0, q2)
-    const df q1 = df_mul_f(df_mul(g1, g1), 6.f);
+    const df2 Q = df2_norm(df2_square(df2_quot_f(f2(m), T)));            // (q0, q2)
+    const df q1 = df_norm(df_scale(df_square(df_quot_f(m, t1)), 6.f));
     const df2 Q1 = df2_make(q1, q1);
-    const df2 W2 = df2_mul_f(df2_swap(Q), f2(3.f));                      // (3 q2, 3 q0)
-    const df2 P0 = df2_add_fast(df2_mul_f(X1, f2(5.f)), df2_mul_pow2(X0, f2(-2.f)));
-    const df2 P1 = df2_add_fast(X1, df2_mul_pow2(X2, f2(2.f)));
-    const df2 P2 = df2_add_fast(df2_mul_pow2(X2, f2(4.f)), df2_neg(X3));
-    const df2 num = df2_add_fast(df2_add_fast(df2_mul(Q, P0), df2_mul(Q1, P1)), df2_mul(W2, P2));
-    const df2 den = df2_mul_f(df2_add_fast(df2_add_fast(Q, Q1), W2), f2(6.f));
-    return df2_div(num, den);   // (increment at c+1/2, increment at c-1/2)
+    const df2 W2 = df2_scale(df2_swap(Q), f2(3.f));                      // (3 q2, 3 q0)
+    const df2 P0 = df2_sum(df2_scale(X1, f2(5.f)), df2_mul_pow2(X0, f2(-2.f)));
+    const df2 P1 = df2_sum(X1, df2_mul_pow2(X2, f2(2.f)));
+    const df2 P2 = df2_sum(df2_mul_pow2(X2, f2(4.f)), df2_neg(X3));
+    const df2 num = df2_sum(df2_sum(df2_prod(Q, P0), df2_prod(Q1, P1)), df2_prod(W2, P2));
+    const df2 den = df2_scale(df2_sum(df2_sum(Q, Q1), W2), f2(6.f));
+    return df2_quot(num, den);   // (increment at c+1/2, increment at c-1/2)
 }
 
 __device__ __forceinline__ void weno5_increments_df(const df (&D)[4], df eps34, df& iR, df& iL) {
@@ -143,14 +144,13 @@ __device__ __forceinline__ void weno5_edges(float vc, const float D[4], float ep
 __device__ __forceinline__ df2 weno3_increments_pair(double a, double b, df E) {
     const df A = df_from_double(a), Bd = df_from_double(b);
     const df2 X = df2_make(A, df_neg(Bd)), Y = df2_make(Bd, df_neg(A));
-    const df2 T = df2_add_fast(df2_make(E, E), df2_mul(df2_make(A, Bd), df2_make(A, Bd)));   // (t0, t1)
+    const df2 T = df2_sum(df2_square(df2_make(A, Bd)), df2_make(E, E));   // (t0, t1)
     const float m = fminf(T.hi.x, T.hi.y);
-    const df2 G = df2_div_f(f2(m), T);
-    const df2 S = df2_mul(G, G);                                     // (s0, s1)
+    const df2 S = df2_norm(df2_square(df2_quot_f(f2(m), T)));        // (s0, s1)
     const df2 S2 = df2_mul_pow2(df2_swap(S), f2(2.f));               // (2 s1, 2 s0)
-    const df2 num = df2_add_fast(df2_mul(S, X), df2_mul(S2, Y));
-    const df2 den = df2_mul_pow2(df2_add_fast(S, S2), f2(2.f));
-    return df2_div(num, den);
+    const df2 num = df2_sum(df2_prod(S, X), df2_prod(S2, Y));
+    const df2 den = df2_mul_pow2(df2_sum(S, S2), f2(2.f));
+    return df2_quot(num, den);
 }
 __device__ __forceinline__ void weno3_edges(double vc, double a, double b, double eps, double& eR, double& eL) {
     const df2 I = weno3_increments_pair(a, b, df_from_double(eps));
@@ -204,28 +204,26 @@ __device__ __forceinline__ df2 weno5_increments_nu_pair(const double D[4], df e,
     const df d2 = df_from_double(D[2]), d3 = df_from_double(D[3]);
     auto C = [&](int kx, int ky) { return df2_make(grid_df(row, kx), grid_df(row, ky)); };
     const df2 Dlo = df2_make(d0, d2), Dhi = df2_make(d1, d3);
-    const df2 Slo = df2_mul(Dlo, Dlo), Shi = df2_mul(Dhi, Dhi);   // (S0, S2), (S1, S3)
-    const df2 X = df2_mul(Dlo, Dhi);                               // (D0 D1, D2 D3)
-    const df2 B = df2_add_fast(df2_add_fast(df2_mul(C(18, 24), Slo), df2_mul(C(19, 25), X)),
-                               df2_mul(C(20, 26), Shi));           // (b0, b2)
-    const df b1 = df_add_fast(df_add_fast(df_mul(grid_df(row, 21), df2_x(Shi)), df_mul(grid_df(row, 22), df_mul(d1, d2))),
-                              df_mul(grid_df(row, 23), df2_y(Slo)));
-    const df2 T = df2_add_fast(df2_make(e, e), B);                 // (t0, t2)
-    const df t1 = df_add_fast(e, b1);
+    const df2 Slo = df2_square(Dlo), Shi = df2_square(Dhi);   // (S0, S2), (S1, S3)
+    const df2 X = df2_prod(Dlo, Dhi);                          // (D0 D1, D2 D3)
+    const df2 B = df2_sum(df2_sum(df2_prod(C(18, 24), Slo), df2_prod(C(19, 25), X)),
+                          df2_prod(C(20, 26), Shi));           // (b0, b2)
+    const df b1 = df_sum(df_sum(df_prod(grid_df(row, 21), df2_x(Shi)), df_prod(grid_df(row, 22), df_prod(d1, d2))),
+                         df_prod(grid_df(row, 23), df2_y(Slo)));
+    const df2 T = df2_sum(B, df2_make(e, e));                  // (t0, t2)
+    const df t1 = df_sum(b1, e);
     const float m = fminf(T.hi.x, fminf(t1.hi, T.hi.y));
-    const df2 G = df2_div_f(f2(m), T);
-    const df2 Q = df2_mul(G, G);                                   // (q0, q2)
-    const df g1 = df_div_f(m, t1);
-    const df q1 = df_mul(g1, g1);
-    const df2 P0 = df2_add_fast(df2_mul(C(0, 6), df2_make(d0, d0)), df2_mul(C(1, 7), df2_make(d1, d1)));
-    const df2 P1 = df2_add_fast(df2_mul(C(2, 8), df2_make(d1, d1)), df2_mul(C(3, 9), df2_make(d2, d2)));
-    const df2 P2 = df2_add_fast(df2_mul(C(4, 10), df2_make(d2, d2)), df2_mul(C(5, 11), df2_make(d3, d3)));
-    const df2 W0 = df2_mul(C(12, 15), df2_make(df2_x(Q), df2_x(Q)));
-    const df2 W1 = df2_mul(C(13, 16), df2_make(q1, q1));
-    const df2 W2 = df2_mul(C(14, 17), df2_make(df2_y(Q), df2_y(Q)));
-    const df2 num = df2_add_fast(df2_add_fast(df2_mul(W0, P0), df2_mul(W1, P1)), df2_mul(W2, P2));
-    const df2 den = df2_add_fast(df2_add_fast(W0, W1), W2);
-    return df2_div(num, den);   // (increment at c+1/2, increment at c-1/2)
+    const df2 Q = df2_norm(df2_square(df2_quot_f(f2(m), T)));  // (q0, q2)
+    const df q1 = df_norm(df_square(df_quot_f(m, t1)));
+    const df2 P0 = df2_sum(df2_prod(C(0, 6), df2_make(d0, d0)), df2_prod(C(1, 7), df2_make(d1, d1)));
+    const df2 P1 = df2_sum(df2_prod(C(2, 8), df2_make(d1, d1)), df2_prod(C(3, 9), df2_make(d2, d2)));
+    const df2 P2 = df2_sum(df2_prod(C(4, 10), df2_make(d2, d2)), df2_prod(C(5, 11), df2_make(d3, d3)));
+    const df2 W0 = df2_prod(C(12, 15), df2_make(df2_x(Q), df2_x(Q)));
+    const df2 W1 = df2_prod(C(13, 16), df2_make(q1, q1));
+    const df2 W2 = df2_prod(C(14, 17), df2_make(df2_y(Q), df2_y(Q)));
+    const df2 num = df2_sum(df2_sum(df2_prod(W0, P0), df2_prod(W1, P1)), df2_prod(W2, P2));
+    const df2 den = df2_sum(df2_sum(W0, W1), W2);
+    return df2_quot(num, den);   // (increment at c+1/2, increment at c-1/2)
 }
 template <class Col>
 __device__ __forceinline__ void weno5_edges_nu(float vc, const float D[4], float eps, const Col& row,
