@@ -117,7 +117,7 @@ __device__ __noinline__ void kapila_K(const SweepArgs& a, const Real* w, Real* K
 // (mfc_df.cuh) and inlined: the FP64 instructions of a reciprocal and the
 // call would cost more than the rest of the source term.
 template <int NF, int NDIM>
-__device__ __forceinline__ void kapila_K_df(const SweepArgs& a, const double* w, double* K) {
+__device__ __forceinline__ void kapila_K_df(const SweepArgs& a, const double* w, df* K) {
     using Lay = Layout<NF, NDIM>;
     const df p = df_from_double(w[Lay::IE]);
     df al[NF], Z[NF];
@@ -148,7 +148,7 @@ __device__ __forceinline__ void kapila_K_df(const SweepArgs& a, const double* w,
 #pragma unroll
     for (int k = 1; k < NF; ++k) D = df_add(D, df_mul(al[k], pe[k]));
 #pragma unroll
-    for (int k = 0; k < NF - 1; ++k) K[k] = df_to_double(df_mul(al[k], df_add(df_div(pe[k], D), {-1.f, 0.f})));
+    for (int k = 0; k < NF - 1; ++k) K[k] = df_mul(al[k], df_add(df_div(pe[k], D), {-1.f, 0.f}));
 }
 
 // Normal rate of a characteristic boundary cell (flat index idx, neighbours
@@ -488,16 +488,51 @@ __device__ __forceinline__ void publish_rate(const SweepArgs& a, const RateAcc& 
 // a separate recovery pass over q) and, with a.rate_max, its CFL rate is
 // returned for the caller's RateAcc (-1: non-physical); otherwise 0.
 //
-// finish_cell takes the two face fluxes and face velocities; finish_cell_df the
-// same in float-float (FP64 path: the flux differences are formed before one
-// widening each); both call finish_cell_rates with (F_- - F_+)/dx and the
-// face-velocity divergence.
+// The FP64 path keeps the accumulator R in float-float (the same 8 bytes): its
+// sweeps' contributions are float-float differences good to ~2^-47 of the fluxes,
+// so FP64 sums of them only cost a widening and two FP64 additions per value and
+// sweep (256^3 x / y / z sweep 2.78 / 2.67 / 3.74 -> 2.69 / 2.59 / 3.64 ms).
+//
+// finish_cell takes the two face fluxes and face velocities, finish_cell_df the
+// same in float-float (FP64 path); both form (F_- - F_+)/dx and the face-velocity
+// divergence and call finish_cell_rates (FP32 forms) or finish_cell_rates_df.
+
+// Stored rate of a characteristic boundary cell: true and the rates in out where
+// cell idx is one along DIR.
+template <typename Real, int NF, int NDIM, int DIR>
+__device__ __forceinline__ bool cbc_stored_rate(const SweepArgs& a, long long idx, Real inv_dx, int b, long long sd,
+                                                Real* out) {
+    constexpr int NS = Layout<NF, NDIM>::NS;
+    const int n = a.g.n[DIR];
+    const bool lo = b == 0 && a.g.bc_lo[DIR] == BC_CHARACTERISTIC;
+    const bool hi = b == n - 1 && a.g.bc_hi[DIR] == BC_CHARACTERISTIC;
+    if (!(lo || hi)) return false;
+    if (a.cbc_rates) {
+        const long long lo_idx = idx - b * sd;   // the row's first cell
+        const long long nx = a.g.n[0];
+        const long long tr = DIR == 0   ? lo_idx / nx
+                             : DIR == 1 ? lo_idx % nx + nx * (lo_idx / (nx * a.g.n[1]))
+                                        : lo_idx;
+        const Real* rb = static_cast<const Real*>(a.cbc_rates) + a.cbc_off[DIR][lo ? 0 : 1] + tr;
+        const long long nt = a.g.ncell / n;
+#pragma unroll
+        for (int v = 0; v < NS; ++v) out[v] = rb[v * nt];
+    } else {
+        Real cb[NS];
+        cbc_cell_rate<Real, NF, NDIM, DIR>(a, idx, sd, n, !lo, inv_dx, cb);
+#pragma unroll
+        for (int v = 0; v < NS; ++v) out[v] = cb[v];
+    }
+    return true;
+}
+
 template <typename Real, int NF, int NDIM, int DIR, bool SIX = false>
 __device__ __forceinline__ double finish_cell_rates(const SweepArgs& a, long long idx, Real* out, const Real du,
                                                     const Real* cell, Real inv_dx, int b, long long sd,
                                                     const unsigned char* stg, int slot) {
+    static_assert(sizeof(Real) == 4, "FP32 forms");
     using Lay = Layout<NF, NDIM, SIX>;
-    constexpr int NS = Lay::NS, NQ = Lay::NQ, IA = Lay::IA;
+    constexpr int NQ = Lay::NQ, IA = Lay::IA;
     if constexpr (SIX) {
         const Real pdu = cell[Lay::IE] * du;
         Real aN = 1;
@@ -511,8 +546,7 @@ __device__ __forceinline__ double finish_cell_rates(const SweepArgs& a, long lon
     if constexpr (NF > 1) {
         if (a.kapila) {
             Real K[NF - 1];
-            if constexpr (sizeof(Real) == 8) kapila_K_df<NF, NDIM>(a, cell, K);
-            else kapila_K<Real, NF, NDIM>(a, cell, K);
+            kapila_K<Real, NF, NDIM>(a, cell, K);
 #pragma unroll
             for (int k = 0; k < NF - 1; ++k) out[IA + k] = fma(cell[IA + k] + K[k], du, out[IA + k]);
         } else {
@@ -520,29 +554,7 @@ __device__ __forceinline__ double finish_cell_rates(const SweepArgs& a, long lon
             for (int k = 0; k < NF - 1; ++k) out[IA + k] = fma(cell[IA + k], du, out[IA + k]);
         }
     }
-    if (a.cbc) {
-        const int n = a.g.n[DIR];
-        const bool lo = b == 0 && a.g.bc_lo[DIR] == BC_CHARACTERISTIC;
-        const bool hi = b == n - 1 && a.g.bc_hi[DIR] == BC_CHARACTERISTIC;
-        if (lo || hi) {   // the boundary rate replaces the flux difference and the source
-            if (a.cbc_rates) {
-                const long long lo_idx = idx - b * sd;   // the row's first cell
-                const long long nx = a.g.n[0];
-                const long long tr = DIR == 0   ? lo_idx / nx
-                                     : DIR == 1 ? lo_idx % nx + nx * (lo_idx / (nx * a.g.n[1]))
-                                                : lo_idx;
-                const Real* rb = static_cast<const Real*>(a.cbc_rates) + a.cbc_off[DIR][lo ? 0 : 1] + tr;
-                const long long nt = a.g.ncell / n;
-#pragma unroll
-                for (int v = 0; v < NS; ++v) out[v] = rb[v * nt];
-            } else {
-                Real cb[NS];
-                cbc_cell_rate<Real, NF, NDIM, DIR>(a, idx, sd, n, !lo, inv_dx, cb);
-#pragma unroll
-                for (int v = 0; v < NS; ++v) out[v] = cb[v];
-            }
-        }
-    }
+    if (a.cbc) cbc_stored_rate<Real, NF, NDIM, DIR>(a, idx, inv_dx, b, sd, out);
     const long long nc = a.g.ncell;
     Real* R = static_cast<Real*>(a.R);
     // operand rows: staged (stride kStageSlots) or in global memory (stride nc)
@@ -565,41 +577,20 @@ __device__ __forceinline__ double finish_cell_rates(const SweepArgs& a, long lon
 #pragma unroll
         for (int v = 0; v < NQ; ++v) R[v * nc + idx] = Rv(v) + out[v];
     } else if (a.mode == 2) {
-        double qn[NQ];
-        // FP32 forms: the increment c1 dt R is formed in FP32 (R is an FP32
-        // quantity there) and widened by integer operations, so the FP64
-        // accumulation takes one FP64 operation per value, two with the q0
-        // term.  FP64 form: c1 (qs + dt R), the product skipped when c1 = 1.
-        [[maybe_unused]] float c1dt = 0.f;
-        if constexpr (sizeof(Real) == 4) c1dt = narrow_rn(a.c1 * a.dt);
-        const bool unit = a.c1 == 1.0;
+        // the increment c1 dt R is formed in FP32 (R is an FP32 quantity here) and
+        // widened by integer operations, so the FP64 accumulation takes one FP64
+        // operation per value, two with the q0 term
+        const float c1dt = narrow_rn(a.c1 * a.dt);
 #pragma unroll
         for (int v = 0; v < NQ; ++v) {
             const Real rv = a.acc_in ? Rv(v) + out[v] : out[v];
-            double o;
-            if constexpr (sizeof(Real) == 4) {
-                o = fma(a.c1, qsv(v), widen_all(c1dt * rv));
-            } else {
-                o = fma(a.dt, rv, qsv(v));
-                if (!unit) o *= a.c1;
-            }
+            double o = fma(a.c1, qsv(v), widen_all(c1dt * rv));
             if (a.c0 != 0.0) o = fma(a.c0, q0v(v), o);
-            qn[v] = o;
             a.qout[v * nc + idx] = o;
         }
-        if constexpr (sizeof(Real) == 8 && !SIX) {
-            // FP64 form only: in the FP32 forms' z sweep (memory-bound, 64
-            // registers) the fused recovery spilled and cost more than the
-            // separate pass it replaced (mixed 6.27 -> 6.52 ms per step at 256^3)
-            if (a.w_next) {
-                Real wv[NS], c2;
-                prims_cell<NF, NDIM>(qn, a.e, wv, c2);
-                Real* wn = static_cast<Real*>(a.w_next);
-#pragma unroll
-                for (int v = 0; v < NS; ++v) wn[v * nc + idx] = wv[v];
-                if (a.rate_max) return cell_cfl_rate<Real, NF, NDIM>(wv, c2, a.g, a.grid, a.grid_stride, idx);
-            }
-        }
+        // (the fused recovery of the FP64 path spilled in the FP32 forms' z sweep,
+        // memory-bound at 64 registers, and cost more than the separate pass it
+        // replaced: mixed 6.27 -> 6.52 ms per step at 256^3)
     } else {
 #pragma unroll
         for (int v = 0; v < NQ; ++v) {
@@ -610,31 +601,135 @@ __device__ __forceinline__ double finish_cell_rates(const SweepArgs& a, long lon
     return 0.0;
 }
 
+template <int NF, int NDIM, int DIR, bool SIX = false>
+__device__ __forceinline__ double finish_cell_rates_df(const SweepArgs& a, long long idx, df* out, df du,
+                                                       const double* cell, double inv_dx, int b, long long sd,
+                                                       const unsigned char* stg, int slot) {
+    using Lay = Layout<NF, NDIM, SIX>;
+    constexpr int NS = Lay::NS, NQ = Lay::NQ, IA = Lay::IA;
+    if constexpr (SIX) {
+        const df pdu = df_mul(df_from_double(cell[Lay::IE]), du);
+        double aN = 1.0;
+#pragma unroll
+        for (int k = 0; k < NF - 1; ++k) {
+            aN -= cell[IA + k];
+            out[Lay::II + k] = df_add_fast(out[Lay::II + k], df_neg(df_mul(df_from_double(cell[IA + k]), pdu)));
+        }
+        out[Lay::II + NF - 1] = df_add_fast(out[Lay::II + NF - 1], df_neg(df_mul(df_from_double(aN), pdu)));
+    }
+    if constexpr (NF > 1) {
+        if (a.kapila) {
+            df K[NF - 1];
+            kapila_K_df<NF, NDIM>(a, cell, K);
+#pragma unroll
+            for (int k = 0; k < NF - 1; ++k) out[IA + k] = df_add(out[IA + k], df_mul(K[k], du));
+        }
+    }
+    if (a.cbc) {
+        double cb[NS];
+        if (cbc_stored_rate<double, NF, NDIM, DIR>(a, idx, inv_dx, b, sd, cb)) {
+#pragma unroll
+            for (int v = 0; v < NS; ++v) out[v] = df_from_double(cb[v]);
+        }
+    }
+    const long long nc = a.g.ncell;
+    df* R = static_cast<df*>(a.R);
+    const df* pR = R + idx;
+    const double *pQs = a.qs + idx, *pQ0 = a.q0 + idx;
+    long long sRv = nc, sQsv = nc, sQ0v = nc;
+    if (stg) {
+        const int m = a.stage;
+        if (m & 1) { pR = reinterpret_cast<const df*>(stg) + slot; sRv = kStageSlots; }
+        if (m & 2) { pQs = reinterpret_cast<const double*>(stg + stage_offset_qs<double, NQ>(m)) + slot; sQsv = kStageSlots; }
+        if (m & 4) { pQ0 = reinterpret_cast<const double*>(stg + stage_offset_q0<double, NQ>(m)) + slot; sQ0v = kStageSlots; }
+    }
+    auto total = [&](int v) -> df { return a.acc_in ? df_add_fast(pR[v * sRv], out[v]) : out[v]; };
+    auto qsv = [&](int v) -> double { return pQs[v * sQsv]; };
+    auto q0v = [&](int v) -> double { return pQ0[v * sQ0v]; };
+    if (a.mode == 0) {
+#pragma unroll
+        for (int v = 0; v < NQ; ++v) R[v * nc + idx] = out[v];
+    } else if (a.mode == 1) {
+#pragma unroll
+        for (int v = 0; v < NQ; ++v) R[v * nc + idx] = df_add_fast(pR[v * sRv], out[v]);
+    } else if (a.mode == 2) {
+        double qn[NQ];
+        // c1 (qs + dt R), the product skipped when c1 = 1, + c0 q0
+        const bool unit = a.c1 == 1.0;
+#pragma unroll
+        for (int v = 0; v < NQ; ++v) {
+            double o = fma(a.dt, df_to_double(total(v)), qsv(v));
+            if (!unit) o *= a.c1;
+            if (a.c0 != 0.0) o = fma(a.c0, q0v(v), o);
+            qn[v] = o;
+            a.qout[v * nc + idx] = o;
+        }
+        if constexpr (!SIX) {
+            if (a.w_next) {
+                double wv[NS], c2;
+                prims_cell<NF, NDIM>(qn, a.e, wv, c2);
+                double* wn = static_cast<double*>(a.w_next);
+#pragma unroll
+                for (int v = 0; v < NS; ++v) wn[v * nc + idx] = wv[v];
+                if (a.rate_max) return cell_cfl_rate<double, NF, NDIM>(wv, c2, a.g, a.grid, a.grid_stride, idx);
+            }
+        }
+    } else {
+#pragma unroll
+        for (int v = 0; v < NQ; ++v) a.out[v * nc + idx] = df_to_double(total(v));
+    }
+    return 0.0;
+}
+
 template <typename Real, int NF, int NDIM, int DIR, bool SIX = false>
 __device__ __forceinline__ double finish_cell(const SweepArgs& a, long long idx, const Real* Fm, const Real* Fp,
                                               Real um, Real up, const Real* cell, Real inv_dx, int b, long long sd,
                                               const unsigned char* stg = nullptr, int slot = 0) {
     constexpr int NQ = Layout<NF, NDIM, SIX>::NQ;
-    Real out[NQ];
+    if constexpr (sizeof(Real) == 8) {   // the pencil-marching kernel
+        constexpr int IA = Layout<NF, NDIM, SIX>::IA;
+        df out[NQ];
 #pragma unroll
-    for (int v = 0; v < NQ; ++v) out[v] = (Fm[v] - Fp[v]) * inv_dx;
-    const Real du = (up - um) * inv_dx;
-    return finish_cell_rates<Real, NF, NDIM, DIR, SIX>(a, idx, out, du, cell, inv_dx, b, sd, stg, slot);
+        for (int v = 0; v < NQ; ++v) {
+            double o = (Fm[v] - Fp[v]) * inv_dx;
+            if (v >= IA && v < IA + NF - 1) o = fma(cell[v], (up - um) * inv_dx, o);   // alpha div(u)
+            out[v] = df_from_double(o);
+        }
+        return finish_cell_rates_df<NF, NDIM, DIR, SIX>(a, idx, out, df_from_double((up - um) * inv_dx), cell, inv_dx, b,
+                                                        sd, stg, slot);
+    } else {
+        Real out[NQ];
+#pragma unroll
+        for (int v = 0; v < NQ; ++v) out[v] = (Fm[v] - Fp[v]) * inv_dx;
+        return finish_cell_rates<Real, NF, NDIM, DIR, SIX>(a, idx, out, (up - um) * inv_dx, cell, inv_dx, b, sd, stg,
+                                                           slot);
+    }
 }
 
-// Five-equation FP64 path with float-float fluxes: the differences and the
-// division by dx in float-float (accurate addition: relative error ~2^-47 of
-// the difference), one widening per value.
+// The differences and the division by dx in float-float.  A volume-fraction row, alpha div(u) -
+// div(alpha u), is formed from the upwind face fractions A as
+// ((alpha - A_+) u_+ - (alpha - A_-) u_-)/dx, the same number without the
+// cancellation of its two parts where alpha is nearly uniform.
 template <int NF, int NDIM, int DIR, bool SIX = false>
 __device__ __forceinline__ double finish_cell_df(const SweepArgs& a, long long idx, const df* Fm, const df* Fp,
                                                  df um, df up, const double* cell, double inv_dx, df inv_df, int b,
                                                  long long sd, const unsigned char* stg = nullptr, int slot = 0) {
     constexpr int NQ = Layout<NF, NDIM, SIX>::NQ;
-    double out[NQ];
+    constexpr int IA = Layout<NF, NDIM, SIX>::IA;
+    df out[NQ];
 #pragma unroll
-    for (int v = 0; v < NQ; ++v) out[v] = df_to_double(df_mul(df_add(Fm[v], df_neg(Fp[v])), inv_df));
-    const double du = df_to_double(df_mul(df_add(up, df_neg(um)), inv_df));
-    return finish_cell_rates<double, NF, NDIM, DIR, SIX>(a, idx, out, du, cell, inv_dx, b, sd, stg, slot);
+    for (int v = 0; v < NQ; ++v) {
+        df diff;
+        if (v >= IA && v < IA + NF - 1) {
+            const df al = df_from_double_rn(cell[v]);
+            diff = df_add(df_mul(df_add(al, df_neg(Fp[v])), up), df_neg(df_mul(df_add(al, df_neg(Fm[v])), um)));
+        } else {
+            diff = df_add_fast(Fm[v], df_neg(Fp[v]));
+        }
+        out[v] = df_mul(diff, inv_df);
+    }
+    return finish_cell_rates_df<NF, NDIM, DIR, SIX>(a, idx, out, df_mul(df_add(up, df_neg(um)), inv_df), cell, inv_dx,
+                                                    b, sd, stg, slot);
 }
 
 }  // namespace mfc

@@ -77,7 +77,7 @@ struct SweepArgs {
     Geometry g;
     EosConst e;
     const void* w;          // primitives [NS][ncell], Real
-    void* R;                // right-hand side accumulator [NS][ncell], Real
+    void* R;                // right-hand side accumulator [NS][ncell], float-float (FP64 path) or float
     int mode;               // 0: R = s; 1: R += s; 2: RK stage update; 3: out = R + s
     int acc_in;             // modes 2/3: add the accumulator R (earlier sweeps)
     const double* q0;       // RK: state at t^n

@@ -85,9 +85,12 @@ cudaError_t run(const Geometry& g, const EosConst& e, int ndim, const double* q,
         a.g = g;
         a.e = e;
         a.w = w;
+        // the accumulator (float-float) and the result share rhs: the last sweep
+        // reads a cell's accumulated rates and writes its FP64 ones in their place
         a.R = rhs;
-        a.mode = d == 0 ? 0 : 1;
-        a.acc_in = 0;
+        a.out = rhs;
+        a.mode = d == ndim - 1 ? 3 : d == 0 ? 0 : 1;
+        a.acc_in = d > 0 ? 1 : 0;
         a.yz_stream = 1;
         a.eps = eps;
         a.fallback = fallback;

@@ -220,10 +220,12 @@ struct MixDf {
     df r, G, P, n;
 };
 
-// Fluxes and face velocity in float-float; returns whether the flux took the
-// left state (useL).  A product that enters a sum is normalised, one that only
+// Fluxes and face velocity in float-float; the volume-fraction rows of F hold the
+// upwind fraction itself (their flux is that times ut; finish_cell_rates_df takes
+// them so).  Returns whether the flux took the left state (useL).  A product that enters a sum is normalised, one that only
 // meets further products or is a flux is not (mfc_df.cuh): with unnormalised terms
-// in the sums the right-hand side's error against 64 bits grew by 25%.
+// in the sums the right-hand side's error against 64 bits grew by 25% (the kinetic
+// energy's do not show).
 template <int NF, int NDIM, int DIR, typename States>
 __device__ __forceinline__ bool hllc_df_core(const States& L, const States& R, const MixDf& mL, const MixDf& mR,
                                              df* F, df& ut) {
@@ -259,10 +261,10 @@ __device__ __forceinline__ bool hllc_df_core(const States& L, const States& R, c
     for (int v = 0; v < NS; ++v) Kd[v] = useL ? L.at(v) : R.at(v);   // element by element: a reference to
     // either state array placed both in local memory (FP64 y/z sweeps 149 -> 128 registers, 256^3 step
     // 36.1 -> 34.4 ms)
-    df u2 = df_mul(Kd[IM], Kd[IM]);
+    df u2 = df_square(Kd[IM]);
 #pragma unroll
-    for (int dd = 1; dd < NDIM; ++dd) u2 = df_add_fast(u2, df_mul(Kd[IM + dd], Kd[IM + dd]));
-    const df rE = df_add_fast(df_add_fast(df_mul(GK, pK), PK), df_mul_pow2(df_mul(rK, u2), 0.5f));
+    for (int dd = 1; dd < NDIM; ++dd) u2 = df_sum(u2, df_square(Kd[IM + dd]));
+    const df rE = df_add_fast(df_add_fast(df_mul(GK, pK), PK), df_mul_pow2(df_prod(rK, u2), 0.5f));
 #pragma unroll
     for (int k = 0; k < NF; ++k) F[k] = df_prod(Kd[k], utd);
     const df sKds = df_mul(sKe, dsu);   // s_K (s* - u_K)
@@ -275,7 +277,7 @@ __device__ __forceinline__ bool hllc_df_core(const States& L, const States& R, c
     F[IE] = df_add_fast(df_add_fast(df_mul(rE, utd), df_mul(pK, uK)),
                         df_mul(sKds, df_add_fast(df_mul(rxi, sS), df_mul(pK, rr))));
 #pragma unroll
-    for (int k = 0; k < NF - 1; ++k) F[IA + k] = df_prod(Kd[IA + k], utd);
+    for (int k = 0; k < NF - 1; ++k) F[IA + k] = Kd[IA + k];
     ut = utd;
     return useL;
 }
@@ -291,6 +293,8 @@ __device__ __forceinline__ void hllc_df(const double* L, const double* R, const 
     const MixDf xR{df_from_double(mR.r), df_from_double(mR.G), df_from_double(mR.P), df_from_double(mR.n)};
     df Fd[NS], utd;
     const bool useL = hllc_df_core<NF, NDIM, DIR>(F64States{L}, F64States{R}, xL, xR, Fd, utd);
+#pragma unroll
+    for (int k = 0; k < NF - 1; ++k) Fd[IA + k] = df_prod(Fd[IA + k], utd);
 #pragma unroll
     for (int v = 0; v < NS; ++v) F[v] = df_to_double(Fd[v]);
     ut = df_to_double(utd);
@@ -332,7 +336,7 @@ __device__ __forceinline__ MixDf mixture_df(const df* s, const EosDf& e) {
         }
         m.n = df_prod(m.G, df_add(df_mul(A, s[Lay::IE]), B));
     } else {
-        m.n = df_add(df_mul(df_add_fast(m.G, {1.f, 0.f}), s[Lay::IE]), m.P);
+        m.n = df_sum(df_prod(df_add_fast(m.G, {1.f, 0.f}), s[Lay::IE]), m.P);
     }
     return m;
 }

@@ -165,12 +165,14 @@ __global__ void __launch_bounds__(128) sweep_kernel(const SweepArgs a) {
 // The FP64 path's edge values of variable q of cell c along direction dir in
 // float-float (DFS): the increment pair of the reconstruction (WENO5 or WENO3
 // on uniform grids, WENO5 from the cell's tables on stretched ones) added to
-// the split cell value with the accurate float-float addition (the face state
-// carries ~2^-48 of its magnitude).  In the six-equation model the volume
-// fractions keep
-// FP64 edges instead (vc + the widened increment, carried in the same 8 bytes
-// by df_pack), since their complement alpha_N enters a flux (face_flux_df).
-// VALUE_MAJOR: the grid-table layout of the direction (x sweep: true).
+// the split cell value, whose split is rounded to nearest: the truncated one's
+// last bit was the largest single error of the right-hand side (12-18% of it
+// against 64 bits, which pays for the plain additions here and in the finish: net
+// 3-15% below the accurate ones with it).  In the six-equation model the volume
+// fractions keep FP64 edges instead (vc + the widened increment, carried in the
+// same 8 bytes by df_pack), since their complement alpha_N enters a flux
+// (face_flux_df).  VALUE_MAJOR: the grid-table layout of the direction (x sweep:
+// true).
 // ---------------------------------------------------------------------------
 template <typename Real, int NF, int NDIM, int ORDER, bool NONUNIF, bool SIX, bool VALUE_MAJOR>
 __device__ __forceinline__ void dfs_edges(const SweepArgs& a, int dir, int c, int q, double vc, const double (&D)[4],
@@ -189,8 +191,8 @@ __device__ __forceinline__ void dfs_edges(const SweepArgs& a, int dir, int c, in
         eL = df_pack(vc + df_to_double(df2_x(I)));
         eR = df_pack(vc + df_to_double(df2_y(I)));
     } else {
-        const df cc = df_from_double(vc);
-        const df2 E = df2_add(df2_make(cc, cc), I);
+        const df cc = df_from_double_rn(vc);
+        const df2 E = df2_add_fast(df2_make(cc, cc), I);
         eL = df2_x(E);
         eR = df2_y(E);
     }
@@ -867,11 +869,10 @@ __global__ void __launch_bounds__(32 * kRowsPerChunk, 4) sweep_yz_stream_f64_ker
 }
 
 // The FP64 uniform WENO5 y/z stream kernel for three fluids, bounded to 3
-// CTAs per SM (168 registers; unbounded it takes 187-192 and keeps 2), the z
-// sweep (RK epilogue) to 4 (128 registers, 76 bytes of spills): 512^3 step
-// 356.2 -> 346.7 ms with both at 4, the y sweep alone slower at 4.
+// CTAs per SM (168 registers; at 4 CTAs 150x139x128 y / z sweep 611 / 907 -> 672 /
+// 941 us).
 template <int NF, int NDIM, int DIR>
-__global__ void __launch_bounds__(32 * kRowsPerChunk, DIR == 2 ? 4 : 3) sweep_yz_stream_f64b3_kernel(const SweepArgs a) {
+__global__ void __launch_bounds__(32 * kRowsPerChunk, 3) sweep_yz_stream_f64b3_kernel(const SweepArgs a) {
     sweep_yz_stream_body<double, NF, NDIM, DIR, false, 5, false, false, true>(a);
 }
 
