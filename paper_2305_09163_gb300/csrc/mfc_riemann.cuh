@@ -430,9 +430,11 @@ __device__ __forceinline__ void face_flux(const SweepArgs& a, const EosR<Real>& 
 // edges (df_pack): alpha_N = 1 - sum_k alpha_k is formed in FP64, since where
 // phase N is a trace (alpha_N ~ 1e-6) the subtraction cancels and a
 // float-float alpha_k (~2^-48 of 1) would leave alpha_N ~3e-9 relative error.
-template <int NF, int NDIM, int DIR, bool SIX = false>
-__device__ __forceinline__ void face_flux_df(const SweepArgs& a, const df* eLs, const df* eRs,
-                                             const double* cl, const double* cr, df* F, df& ut) {
+// cells(v, side) gives variable v of the left (0) or right (1) cell; it is called
+// only where a face falls back, so the two cells' states need not be at hand.
+template <int NF, int NDIM, int DIR, bool SIX = false, typename Cells>
+__device__ __forceinline__ void face_flux_df(const SweepArgs& a, const df* eLs, const df* eRs, const Cells& cells,
+                                             df* F, df& ut) {
     using Lay = Layout<NF, NDIM>;
     constexpr int NS = Lay::NS;
     const EosDf& e = a.ed;
@@ -459,14 +461,14 @@ __device__ __forceinline__ void face_flux_df(const SweepArgs& a, const df* eLs, 
         count_fallback(a.fallback_count);
 #pragma unroll
         for (int v = 0; v < NS; ++v) {
-            sl[v] = df_from_double(cl[v]);
-            sr[v] = df_from_double(cr[v]);
-        }
-        if constexpr (SIX) {
-#pragma unroll
-            for (int k = 0; k < NF - 1; ++k) {
-                aL[k] = cl[Lay::IA + k];
-                aR[k] = cr[Lay::IA + k];
+            const double cl = cells(v, 0), cr = cells(v, 1);
+            sl[v] = df_from_double(cl);
+            sr[v] = df_from_double(cr);
+            if constexpr (SIX) {
+                if (v >= Lay::IA && v < Lay::IA + NF - 1) {
+                    aL[v - Lay::IA] = cl;
+                    aR[v - Lay::IA] = cr;
+                }
             }
         }
         mL = mixture_df<NF, NDIM, SIX>(sl, e);

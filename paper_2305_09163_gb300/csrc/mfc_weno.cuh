@@ -141,8 +141,7 @@ __device__ __forceinline__ void weno5_edges(float vc, const float D[4], float ep
 // ---------------------------------------------------------------------------
 // The two WENO3 increments (c+1/2 in lane x, c-1/2 in lane y): lane y evaluates
 // the c+1/2 formula on the mirrored differences (-b, -a).
-__device__ __forceinline__ df2 weno3_increments_pair(double a, double b, df E) {
-    const df A = df_from_double(a), Bd = df_from_double(b);
+__device__ __forceinline__ df2 weno3_increments_pair(df A, df Bd, df E) {
     const df2 X = df2_make(A, df_neg(Bd)), Y = df2_make(Bd, df_neg(A));
     const df2 T = df2_sum(df2_square(df2_make(A, Bd)), df2_make(E, E));   // (t0, t1)
     const float m = fminf(T.hi.x, T.hi.y);
@@ -153,7 +152,7 @@ __device__ __forceinline__ df2 weno3_increments_pair(double a, double b, df E) {
     return df2_quot(num, den);
 }
 __device__ __forceinline__ void weno3_edges(double vc, double a, double b, double eps, double& eR, double& eL) {
-    const df2 I = weno3_increments_pair(a, b, df_from_double(eps));
+    const df2 I = weno3_increments_pair(df_from_double(a), df_from_double(b), df_from_double(eps));
     eL = vc + df_to_double(df2_x(I));
     eR = vc + df_to_double(df2_y(I));
 }
@@ -196,12 +195,11 @@ __device__ __forceinline__ df grid_df(const Col& row, int k) {
 }
 
 template <class Col>
-__device__ __forceinline__ df2 weno5_increments_nu_pair(const double D[4], df e, const Col& row) {
+__device__ __forceinline__ df2 weno5_increments_nu_pair(const df (&D)[4], df e, const Col& row) {
     // the two edges side by side in packed FP32 instructions: lane x the c+1/2
     // edge (coefficients 0-5, 12-14), lane y the c-1/2 edge (6-11, 15-17); the
     // smoothness indicators b0 and b2 side by side, b1 alone
-    const df d0 = df_from_double(D[0]), d1 = df_from_double(D[1]);
-    const df d2 = df_from_double(D[2]), d3 = df_from_double(D[3]);
+    const df d0 = D[0], d1 = D[1], d2 = D[2], d3 = D[3];
     auto C = [&](int kx, int ky) { return df2_make(grid_df(row, kx), grid_df(row, ky)); };
     const df2 Dlo = df2_make(d0, d2), Dhi = df2_make(d1, d3);
     const df2 Slo = df2_square(Dlo), Shi = df2_square(Dhi);   // (S0, S2), (S1, S3)
