@@ -415,13 +415,20 @@ template <typename Real, int NF, int NDIM>
 __device__ __forceinline__ double cell_cfl_rate(const Real* wv, Real c2, const Geometry& g, const float* const* grid,
                                                 const int* grid_stride, long long i) {
     constexpr int IM = Layout<NF, NDIM>::IM;
-    Real us = 0;
-#pragma unroll
-    for (int d = 0; d < NDIM; ++d) us += wv[IM + d];
-    if (!(c2 > (Real)0) || !(c2 - c2 == (Real)0) || !(us - us == (Real)0)) return -1.0;
     Real cs;
-    if constexpr (sizeof(Real) == 8) cs = df_to_double(df_sqrt(df_from_double(c2)));
-    else cs = real_sqrt(c2);
+    if constexpr (sizeof(Real) == 8) {   // the same tests and maxima on the bit patterns: FP64 ones use the FP64 pipe
+        bool ok = positive(c2) && finite_bits(c2);
+#pragma unroll
+        for (int d = 0; d < NDIM; ++d) ok = ok && finite_bits(wv[IM + d]);
+        if (!ok) return -1.0;
+        cs = df_to_double(df_sqrt(df_from_double(c2)));
+    } else {
+        Real us = 0;
+#pragma unroll
+        for (int d = 0; d < NDIM; ++d) us += wv[IM + d];
+        if (!(c2 > (Real)0) || !(c2 - c2 == (Real)0) || !(us - us == (Real)0)) return -1.0;
+        cs = real_sqrt(c2);
+    }
     Real r = 0;
     int ci[3] = {0, 0, 0};
     if (grid[0] || grid[1] || grid[2]) {   // non-uniform: this cell's widths
@@ -435,7 +442,8 @@ __device__ __forceinline__ double cell_cfl_rate(const Real* wv, Real c2, const G
         const Real inv = !grid[d] ? (Real)g.inv_dx[d]
                          : d == 0 ? grid_inv_dx<true>(grid[d], grid_stride[d], ci[d], Real(0))
                                   : grid_inv_dx<false>(grid[d], grid_stride[d], ci[d], Real(0));
-        r = real_max(r, (fabs(wv[IM + d]) + cs) * inv);
+        if constexpr (sizeof(Real) == 8) r = max_nonneg(r, (fabs(wv[IM + d]) + cs) * inv);
+        else r = real_max(r, (fabs(wv[IM + d]) + cs) * inv);
     }
     return (double)r;
 }
@@ -448,8 +456,8 @@ struct RateAcc {
     double rate = 0.0;
     int bad = 0;
     __device__ __forceinline__ void add(double r) {
-        if (r < 0.0) bad += 1;
-        else rate = fmax(rate, r);
+        if (__double2hiint(r) < 0) bad += 1;   // -1: the only negative value
+        else rate = max_nonneg(rate, r);
     }
 };
 
@@ -654,12 +662,11 @@ __device__ __forceinline__ double finish_cell_rates_df(const SweepArgs& a, long 
         for (int v = 0; v < NQ; ++v) R[v * nc + idx] = df_add_fast(pR[v * sRv], out[v]);
     } else if (a.mode == 2) {
         double qn[NQ];
-        // c1 (qs + dt R), the product skipped when c1 = 1, + c0 q0
-        const bool unit = a.c1 == 1.0;
+        // c1 qs + c0 q0 + c1 dt R, the last product in float-float before it is
+        // widened: one FP64 instruction per value fewer
 #pragma unroll
         for (int v = 0; v < NQ; ++v) {
-            double o = fma(a.dt, df_to_double(total(v)), qsv(v));
-            if (!unit) o *= a.c1;
+            double o = fma(a.c1, qsv(v), df_to_double(df_prod(total(v), a.c1dtd)));
             if (a.c0 != 0.0) o = fma(a.c0, q0v(v), o);
             qn[v] = o;
             a.qout[v * nc + idx] = o;

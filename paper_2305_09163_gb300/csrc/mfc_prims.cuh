@@ -56,8 +56,8 @@ __global__ void __launch_bounds__(256) prims_kernel(const PrimArgs a) {
         for (int v = 0; v < NS; ++v) w[v * nc + i] = wv[v];
         if (RATE) {
             const double r = cell_cfl_rate<Real, NF, NDIM>(wv, c2, a.g, a.grid, a.grid_stride, i);
-            if (r < 0.0) bad += 1;
-            else rate = fmax(rate, r);
+            if (__double2hiint(r) < 0) bad += 1;
+            else rate = max_nonneg(rate, r);
         }
     }
     if (RATE) publish_block_rate(a, rate, bad);
@@ -301,8 +301,8 @@ __global__ void __launch_bounds__(256) relax_prims_kernel(const PrimArgs a, cons
         for (int v = 0; v < NS; ++v) w[v * nc + i] = wv[v];
         if (RATE) {
             const double r = cell_cfl_rate<Real, NF, NDIM>(wv, c2, a.g, a.grid, a.grid_stride, i);
-            if (r < 0.0) bad += 1;
-            else rate = fmax(rate, r);
+            if (__double2hiint(r) < 0) bad += 1;
+            else rate = max_nonneg(rate, r);
         }
     }
     if (RATE) publish_block_rate(a, rate, bad);

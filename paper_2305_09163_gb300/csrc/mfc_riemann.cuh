@@ -71,6 +71,12 @@ __device__ __forceinline__ bool positive(double x) {        // x > 0
     const unsigned long long u = (unsigned long long)__double_as_longlong(x);
     return u - 1ULL < 0x7FF0000000000000ULL;
 }
+__device__ __forceinline__ bool finite_bits(double x) {
+    return ((unsigned)__double2hiint(x) & 0x7FF00000u) != 0x7FF00000u;
+}
+__device__ __forceinline__ double max_nonneg(double a, double b) {   // a, b >= 0: ordered as integers
+    return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
+}
 __device__ __forceinline__ bool nonneg(float x) { return x >= 0.f; }
 __device__ __forceinline__ bool unit_interval(float x) { return x >= 0.f && x <= 1.f; }
 __device__ __forceinline__ bool positive(float x) { return x > 0.f; }
