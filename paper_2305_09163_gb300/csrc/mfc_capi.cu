@@ -69,15 +69,14 @@ struct mfc_ctx {
     void* R = nullptr;        // RHS accumulator (double or float)
     void* w = nullptr;        // primitives (double or float)
     void* w2 = nullptr;       // the other primitive buffer: the RK epilogue writes the next stage's here
-    unsigned long long* d_rate = nullptr;  // CFL max (ordered bits)
-    int* d_bad = nullptr;
+    unsigned long long* d_rate = nullptr;  // [0] CFL max (ordered bits), [1] count of non-physical cells (int)
     unsigned long long* d_fallback = nullptr;  // [0] fallback faces, [1] learned-form network rows
     unsigned long long* h_pin = nullptr;   // pinned readback [rate, bad]
     float* mlp = nullptr;         // network parameters, then (at byte kMlpFragOffset) the packed fragments
 
     bool state_set = false;
     bool w_valid = false;     // w holds the primitives of q
-    bool rate_valid = false;  // d_rate / d_bad hold the CFL rate of q (written by the last RK epilogue)
+    bool rate_valid = false;  // d_rate holds the CFL rate of q (written by the last RK epilogue)
     bool dead = false;
     long long launches = 0;
     std::string err;
@@ -107,6 +106,8 @@ mfc_status fail(mfc_ctx* c, mfc_status s, const char* fmt, ...) {
         if (e_ != cudaSuccess)                                                             \
             return fail((ctx), MFC_ERR_CUDA, "%s: %s", #call, cudaGetErrorString(e_));     \
     } while (0)
+
+int* bad_count(const mfc_ctx* c) { return reinterpret_cast<int*>(c->d_rate + 1); }
 
 bool is_f32(const mfc_ctx* c) { return c->precision != MFC_FP64; }
 
@@ -268,7 +269,7 @@ mfc_status run_prims(mfc_ctx* c, const double* src, bool rate, bool relax = fals
     a.q = src;
     a.w = c->w;
     a.rate_max = rate ? c->d_rate : nullptr;
-    a.bad = rate ? c->d_bad : nullptr;
+    a.bad = rate ? bad_count(c) : nullptr;
     for (int d = 0; d < 3; ++d) {   // layouts as mfc_set_grid stores them
         a.grid[d] = c->grid[d];
         a.grid_stride[d] = c->n[d] + 2;
@@ -361,7 +362,8 @@ mfc_status run_cbc(mfc_ctx* c, SweepArgs& a) {
     });
 }
 
-mfc_status run_sweeps(mfc_ctx* c, double* out, const RkStage* rk, void* w_next = nullptr, bool rate = false) {
+mfc_status run_sweeps(mfc_ctx* c, double* out, const RkStage* rk, void* w_next = nullptr, bool rate = false,
+                      bool reset = false) {
     SweepArgs cb{};
     if (has_cbc(c)) {
         cb = base_sweep(c);
@@ -380,6 +382,7 @@ mfc_status run_sweeps(mfc_ctx* c, double* out, const RkStage* rk, void* w_next =
         a.R = c->R;
         const bool last = (d == c->ndim - 1);
         a.acc_in = c->ndim > 1 ? 1 : 0;
+        a.rate_reset = reset && d == 0 ? c->d_rate : nullptr;
         if (last && rk) {
             a.mode = 2;
             a.q0 = rk->q0;
@@ -391,7 +394,7 @@ mfc_status run_sweeps(mfc_ctx* c, double* out, const RkStage* rk, void* w_next =
             a.c1dtd = df_split(rk->c1 * rk->dt);
             a.w_next = w_next;
             a.rate_max = rate ? c->d_rate : nullptr;
-            a.bad = rate ? c->d_bad : nullptr;
+            a.bad = rate ? bad_count(c) : nullptr;
         } else if (last) {
             a.mode = 3;
             a.out = out;
@@ -425,7 +428,6 @@ void free_all(mfc_ctx* c) {
     cudaFree(c->w);
     cudaFree(c->w2);
     cudaFree(c->d_rate);
-    cudaFree(c->d_bad);
     cudaFree(c->d_fallback);
     cudaFree(c->mlp);
     for (int d = 0; d < 3; ++d) cudaFree(c->grid[d]);
@@ -525,8 +527,7 @@ mfc_status mfc_init(mfc_ctx** out, int nx, int ny, int nz, const double lo[3], c
     if ((e = cudaMalloc(&c->q, bytes)) != cudaSuccess || (e = cudaMalloc(&c->q1, bytes)) != cudaSuccess ||
         (e = cudaMalloc(&c->R, wbytes)) != cudaSuccess || (e = cudaMalloc(&c->w, wbytes)) != cudaSuccess ||
         (e = cudaMalloc(&c->w2, wbytes)) != cudaSuccess ||
-        (e = cudaMalloc(&c->d_rate, sizeof(unsigned long long))) != cudaSuccess ||
-        (e = cudaMalloc(&c->d_bad, sizeof(int))) != cudaSuccess ||
+        (e = cudaMalloc(&c->d_rate, 2 * sizeof(unsigned long long))) != cudaSuccess ||
         (e = cudaMalloc(&c->d_fallback, 2 * sizeof(unsigned long long))) != cudaSuccess ||
         (e = cudaMallocHost(&c->h_pin, 2 * sizeof(unsigned long long))) != cudaSuccess) {
         const bool oom = (e == cudaErrorMemoryAllocation);
@@ -727,12 +728,17 @@ mfc_status mfc_step(mfc_ctx* c, double dt) {
     // memory-bound z sweep gains nothing from a fused recovery: they recover
     // separately.
     const bool fused = !c->six && !is_f32(c);
+    // The CFL words of the last stage are cleared by the step's first launch, or
+    // by a memset where that launch publishes to them itself (1D, one stage).
+    bool first = true;
     auto stage = [&](const RkStage& st, bool last) -> mfc_status {
-        if (last && (fused || c->six)) {
-            MFC_CUDA(c, cudaMemsetAsync(c->d_rate, 0, sizeof(unsigned long long), c->stream));
-            MFC_CUDA(c, cudaMemsetAsync(c->d_bad, 0, sizeof(int), c->stream));
+        bool reset = first && (fused || c->six);
+        first = false;
+        if (reset && last && c->ndim == 1 && fused) {
+            MFC_CUDA(c, cudaMemsetAsync(c->d_rate, 0, 2 * sizeof(unsigned long long), c->stream));
+            reset = false;
         }
-        mfc_status r = run_sweeps(c, nullptr, &st, fused ? c->w2 : nullptr, fused && last);
+        mfc_status r = run_sweeps(c, nullptr, &st, fused ? c->w2 : nullptr, fused && last, reset);
         if (r != MFC_OK) return r;
         if (fused) std::swap(c->w, c->w2);
         if (c->six) return run_prims(c, st.qout, last, true);
@@ -776,16 +782,14 @@ mfc_status mfc_cfl_dt(mfc_ctx* c, double cfl, double* dt_out) {
     if (!dt_out || !(cfl > 0.0) || !std::isfinite(cfl)) return fail(c, MFC_ERR_ARG, "bad cfl or NULL dt_out");
     if (!c->state_set) return fail(c, MFC_ERR_STATE_UNSET, "no state set");
     if (!c->rate_valid) {   // else the last RK epilogue computed it for this state
-        MFC_CUDA(c, cudaMemsetAsync(c->d_rate, 0, sizeof(unsigned long long), c->stream));
-        MFC_CUDA(c, cudaMemsetAsync(c->d_bad, 0, sizeof(int), c->stream));
+        MFC_CUDA(c, cudaMemsetAsync(c->d_rate, 0, 2 * sizeof(unsigned long long), c->stream));
         s = run_prims(c, c->q, true);
         if (s != MFC_OK) return s;
         c->w_valid = true;
         c->rate_valid = true;
     }
-    MFC_CUDA(c, cudaMemcpyAsync(&c->h_pin[0], c->d_rate, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
+    MFC_CUDA(c, cudaMemcpyAsync(&c->h_pin[0], c->d_rate, 2 * sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                                 c->stream));
-    MFC_CUDA(c, cudaMemcpyAsync(&c->h_pin[1], c->d_bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     MFC_CUDA(c, cudaStreamSynchronize(c->stream));
     const int bad = *reinterpret_cast<int*>(&c->h_pin[1]);
     double rate;

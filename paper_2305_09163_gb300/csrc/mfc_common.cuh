@@ -85,6 +85,7 @@ struct SweepArgs {
     double* qout;           // RK: output stage state (may alias qs or q0)
     double* out;            // mode 3: float64 right-hand side output
     void* w_next;           // mode 2, optional: primitives of qout [NS][ncell], Real (five-equation models)
+    unsigned long long* rate_reset;  // optional: two words this launch sets to zero (a later one's rate_max and bad)
     unsigned long long* rate_max;  // with w_next, optional: CFL rate of qout, max as ordered bits
     int* bad;               // with rate_max: count of non-physical cells of qout
     double c0, c1, dt;      // RK: qout = c0 q0 + c1 (qs + dt (R + s))
@@ -217,6 +218,16 @@ template <int NF, int NDIM, bool SIX = false> struct Layout {
 __host__ __device__ inline long long stride_of(const Geometry& g, int d) {
     return d == 0 ? 1LL : (d == 1 ? (long long)g.n[0] : (long long)g.n[0] * g.n[1]);
 }
+
+// Programmatic dependent launch: a kernel launched by launch_pdl
+// (mfc_launch.cuh) may be set up while the one ahead of it in the stream still
+// ends, so it calls pdl_wait before its first access to global memory, which
+// returns when the one ahead has ended and its writes are visible (a later
+// kernel's own wait covers all earlier ones, since each ends only after its
+// wait).  No kernel releases its successor early: resident before there was room on
+// every SM, the successor's CTAs crowded onto some (2D 301x201 step of five 530 ->
+// 590 us, RHS of 48x41x33 61 -> 77 us).
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
 
 // Ghost-cell index mapping along one axis (Sec. 3.3).  Valid for i in
 // [-3, n+2] and n >= 3.  Sets *flip for reflective ghosts.

@@ -17,7 +17,7 @@
 #include <cstdint>
 
 #include "../../include/mfc.h"
-#include "mfc_device.cuh"
+#include "mfc_launch.cuh"
 #include "mfc_mlp.cuh"
 
 using namespace mfc;
@@ -343,6 +343,7 @@ __global__ void __launch_bounds__(32 * kReduceWarps) mlp_reduce_kernel(const flo
     __shared__ float sh[kReduceWarps][32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int p = blockIdx.x * 32 + lane;
+    pdl_wait();
     float s = 0.f;
     if (p <= kMlpParams) {
 #pragma unroll 8
@@ -363,6 +364,7 @@ __global__ void mlp_adam_kernel(float* __restrict__ P, const float* __restrict__
                                 float c2) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n) return;
+    pdl_wait();
     const float gi = G[i];
     const float m = b1 * M[i] + (1.f - b1) * gi;
     const float v = b2 * V[i] + (1.f - b2) * gi * gi;
@@ -719,8 +721,7 @@ __global__ void __launch_bounds__(32) mlp_pack_kernel(const float* __restrict__ 
 
 // Host launcher of the partial-gradient sum, used by both gradient entries.
 cudaError_t mfc_launch_mlp_reduce(const float* work, int parts, float* grad, float* loss, cudaStream_t s) {
-    mlp_reduce_kernel<<<(kGradStride + 31) / 32, 32 * kReduceWarps, 0, s>>>(work, parts, grad, loss);
-    return cudaGetLastError();
+    return launch_pdl(mlp_reduce_kernel, (kGradStride + 31) / 32, 32 * kReduceWarps, 0, s, work, parts, grad, loss);
 }
 
 // Host launcher used by mfc_set_mlp: frag holds kMlpFragBytes.
@@ -777,9 +778,10 @@ mfc_status mfc_mlp_adam(float* params, const float* grad, float* m, float* v, in
         return MFC_ERR_ARG;
     const float c1 = (float)(1.0 / (1.0 - std::pow((double)beta1, step)));
     const float c2 = (float)(1.0 / (1.0 - std::pow((double)beta2, step)));
-    mlp_adam_kernel<<<(n + 255) / 256, 256, 0, static_cast<cudaStream_t>(stream)>>>(params, grad, m, v, n, lr, beta1,
-                                                                                  beta2, eps, c1, c2);
-    return cudaGetLastError() == cudaSuccess ? MFC_OK : MFC_ERR_CUDA;
+    return launch_pdl(mlp_adam_kernel, (unsigned)((n + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream), params,
+                      grad, m, v, n, lr, beta1, beta2, eps, c1, c2) == cudaSuccess
+               ? MFC_OK
+               : MFC_ERR_CUDA;
 }
 
 mfc_status mfc_harvest(const double* w_fine, int nxf, int nyf, int nzf, int num_fluids, double weno_eps, double tau,

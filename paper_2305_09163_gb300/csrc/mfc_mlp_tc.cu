@@ -27,6 +27,7 @@
 #include <cstdint>
 
 #include "../../include/mfc.h"
+#include "mfc_launch.cuh"
 #include "mfc_mlp.cuh"
 #include "mfc_tc.cuh"
 
@@ -104,6 +105,7 @@ __device__ void load_weights(unsigned char* sm, int bytes, const float* __restri
     for (int i = threadIdx.x * 16; i < bytes; i += blockDim.x * 16)
         *reinterpret_cast<uint4*>(sm + i) = make_uint4(0u, 0u, 0u, 0u);
     __syncthreads();
+    pdl_wait();   // the parameters may be the kernel ahead's
     for (int i = threadIdx.x; i < kMlpH * kMlpH; i += blockDim.x) {
         const int n = i / kMlpH, k = i % kMlpH;
         put_bf16(sm + FwdLayout::w2, 32, n, k, P[kOffW2 + n * kMlpH + k]);
@@ -403,9 +405,10 @@ mfc_status mfc_mlp_forward_tc(const float* params, const float* x, long long bat
     if (cudaFuncSetAttribute(mlp_forward_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kFwdSmem) !=
         cudaSuccess)
         return MFC_ERR_CUDA;
-    mlp_forward_tc_kernel<<<grid_for(batch, 4), kTile, kFwdSmem, static_cast<cudaStream_t>(stream)>>>(params, x,
-                                                                                                     batch, omega);
-    return cudaGetLastError() == cudaSuccess ? MFC_OK : MFC_ERR_CUDA;
+    return launch_pdl(mlp_forward_tc_kernel, grid_for(batch, 4), kTile, kFwdSmem, static_cast<cudaStream_t>(stream),
+                      params, x, batch, omega) == cudaSuccess
+               ? MFC_OK
+               : MFC_ERR_CUDA;
 }
 
 mfc_status mfc_mlp_grad(const float* params, const float* x, const float* phat, const float* target,
@@ -419,8 +422,9 @@ mfc_status mfc_mlp_grad(const float* params, const float* x, const float* phat, 
         return MFC_ERR_CUDA;
     const unsigned blocks = grid_for(batch, 2);
     static_assert(2LL * 152 * kTcStride <= MFC_MLP_WORK_FLOATS, "workspace holds every CTA's partial");
-    mlp_grad_tc_kernel<<<blocks, kTile, kGradSmem, s>>>(params, x, phat, target, mask, batch, lam, work);
-    if (cudaGetLastError() != cudaSuccess) return MFC_ERR_CUDA;
+    if (launch_pdl(mlp_grad_tc_kernel, blocks, kTile, kGradSmem, s, params, x, phat, target, mask, batch, lam, work) !=
+        cudaSuccess)
+        return MFC_ERR_CUDA;
     return mfc_launch_mlp_reduce(work, (int)blocks, grad, loss, s) == cudaSuccess ? MFC_OK : MFC_ERR_CUDA;
 }
 

@@ -41,6 +41,7 @@ template <typename Real, int NF, int NDIM, bool RATE, bool SIX = false>
 __global__ void __launch_bounds__(256) prims_kernel(const PrimArgs a) {
     using Lay = Layout<NF, NDIM>;
     constexpr int NS = Lay::NS;
+    pdl_wait();
     const long long nc = a.g.ncell;
     double rate = 0.0;
     int bad = 0;
@@ -263,6 +264,7 @@ template <typename Real, int NF, int NDIM, bool RATE>
 __global__ void __launch_bounds__(256) relax_prims_kernel(const PrimArgs a, const RelaxConst c) {
     using Lay = Layout<NF, NDIM, true>;
     constexpr int NS = Lay::NS, NQ = Lay::NQ, IM = Lay::IM, IE = Lay::IE, IA = Lay::IA, II = Lay::II;
+    pdl_wait();
     const long long nc = a.g.ncell;
     double rate = 0.0;
     int bad = 0;

@@ -197,6 +197,12 @@ __device__ __forceinline__ void dfs_edges(const SweepArgs& a, int dir, int c, in
     }
 }
 
+// Clear the CFL words a later launch of this step publishes to (x sweep of the
+// first stage; instead of a memset of its own per step).
+__device__ __forceinline__ void reset_rate(const SweepArgs& a) {
+    if (a.rate_reset && blockIdx.x == 0 && threadIdx.x < 2) a.rate_reset[threadIdx.x] = 0;
+}
+
 // ---------------------------------------------------------------------------
 constexpr int kStreamThreads = 128;
 
@@ -235,6 +241,8 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
     __shared__ Real sh_eRJ[NJ][kStreamThreads];
     __shared__ Real sh_F[NQ + 1][ER];
     df(*dsh_F)[ER] = reinterpret_cast<df(*)[ER]>(sh_F);   // DFS: float-float fluxes
+    pdl_wait();
+    reset_rate(a);
     const Real* __restrict__ w = static_cast<const Real*>(a.w);
     const int n = a.g.n[0];
     const long long rowlen = (long long)n + 2;
@@ -607,6 +615,7 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
     df(*dsh_F)[ER][32] = reinterpret_cast<df(*)[ER][32]>(sh_F);   // DFS: float-float fluxes
     extern __shared__ __align__(16) unsigned char stage_smem[];   // a.stage operands
     static_assert(32 * kRowsPerChunk == kStageSlots, "one staging slot per thread");
+    pdl_wait();
     const Real* __restrict__ w = static_cast<const Real*>(a.w);
     const int lane = threadIdx.x & 31, row = threadIdx.x >> 5;
     // lanes run over the flat transverse plane (x fastest), so only the plane's
