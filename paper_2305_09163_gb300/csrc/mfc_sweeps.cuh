@@ -688,11 +688,13 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
                 staged = a.stage;
                 if (staged) stage_finish_operands<Real, NQ>(a, fidx, stage_smem, threadIdx.x);
             }
-            // FP32 five-equation forms only: measured faster there (mixed 6.46 ->
-            // 6.27, learned 14.2 -> 12.8, mixed stretched 10.3 -> 8.7 ms per step
-            // at 256^3), not for the FP64 stretched-grid (70.3 -> 70.6) or the
-            // six-equation sweeps (mixed 16.9 -> 17.2)
-            if constexpr (sizeof(Real) == 4 && !SIX)
+            // Measured: FP32 five-equation forms (mixed 6.46 -> 6.27, learned 14.2 ->
+            // 12.8, mixed stretched 10.3 -> 8.7 ms per step at 256^3) and FP64 sweeps
+            // that end a stage or stage nothing (256^3 z 3.35 -> 3.29 ms, 3 fluids
+            // 150x139x128 z 843 -> 813 us, stretched 128x120x112 y / z 399 / 512 ->
+            // 383 / 490); not the FP64 y sweep with R staged (2.49 -> 2.51 ms) nor the
+            // six-equation sweeps (mixed 16.9 -> 17.2, FP64 unchanged)
+            if constexpr (!SIX && (sizeof(Real) == 4 || DIR == NDIM - 1 || NONUNIF))
                 prefetch_finish_operands<Real, NQ>(a, fidx, stage_mask(a) & ~staged);
         }
         Real cell[NS], cm1[NS], eL[NS], eR[NS];
