@@ -19,6 +19,15 @@
 //             are dW2, dW1 and dW3; it accumulates in tensor memory over all
 //             tiles of the CTA and is read out once.
 //
+// The gradient keeps [H1 | H2 | X] and [dZ2 | dZ1 | dZ3] in two tiles of 128
+// samples x 80 columns: column ranges of them are the K-major operands of the
+// layers, and read across (MN-major descriptors) they are the transposed operands of
+// the weight chain, which were written out element by element before (136 two-byte
+// stores per sample, four-way bank conflicts, 54% of the shared-memory pipe).  With
+// one accumulator range for all layers a CTA takes 48 KB and 128 tensor-memory
+// columns, so four share an SM and a batch of 65,536 is one tile per CTA; it was two
+// CTAs of two tiles (22 us per gradient, @@ now).
+//
 // Bias gradients and the loss are FP32 sums in registers.  Every wait on the
 // mbarrier is bounded; a wait that gives up sets an error flag (read by
 // mfc_mlp_tc_status), the CTA waits once more for its MMAs, frees its tensor
@@ -53,33 +62,33 @@ constexpr int kXA = kTile * 16 * 2;  // A: X [128][16] (columns >= 5 zero)
 constexpr int kHA = kTile * 32 * 2;  // A: H1, H2 [128][32]
 constexpr int kW3tB = 32 * 16 * 2;   // B: W3^T [n 32][k 16] (k >= 3 zero)
 constexpr int kW2tB = 32 * 32 * 2;   // B: W2^T [n 32][k 32]
-constexpr int kDZ3A = kTile * 16 * 2;
-constexpr int kAW = 128 * kTile * 2;  // A: [dZ2^T; dZ1^T; dZ3^T; 0] [128][batch 128]
-constexpr int kBWN = 80;
-constexpr int kBW = kBWN * kTile * 2;  // B: [H1^T; H2^T; X^T; 0] [80][batch 128]
+constexpr int kCols = 80;                  // columns of the gradient's two sample tiles
+constexpr int kSampleTile = kTile * kCols * 2;
 
 struct FwdLayout {
     static constexpr int w1 = 0, w2 = w1 + kW1B, w3 = w2 + kW2B, x = w3 + kW3B, h1 = x + kXA, h2 = h1 + kHA;
     static constexpr int end = h2 + kHA;
 };
 struct GradLayout {
-    static constexpr int w1 = 0, w2 = w1 + kW1B, w3 = w2 + kW2B, x = w3 + kW3B, h1 = x + kXA, h2 = h1 + kHA;
-    static constexpr int w3t = h2 + kHA, w2t = w3t + kW3tB, dz3 = w2t + kW2tB, dz2 = dz3 + kDZ3A;
-    static constexpr int aw = dz2 + kHA, bw = aw + kAW;
-    static constexpr int end = bw + kBW;
+    static constexpr int w1 = 0, w2 = w1 + kW1B, w3 = w2 + kW2B, w3t = w3 + kW3B, w2t = w3t + kW3tB;
+    // dz: columns dZ2 0-31, dZ1 32-63, dZ3 64-66; act: H1 0-31, H2 32-63, X 64-68; the
+    // rest stays zero.  The weight chain's A has M = 128: its columns past 79 are read
+    // from the rows behind (the last ones from act), into accumulator rows nobody reads.
+    static constexpr int dz = w2t + kW2tB, act = dz + kSampleTile;
+    static constexpr int end = act + kSampleTile;
 };
-// The forward kernel pads its shared memory so that at most four CTAs share an
-// SM (4 x 128 tensor-memory columns); the gradient kernel's 91 KB allows two
-// (2 x 256 columns).
+// Both kernels run four CTAs per SM: 4 x 128 tensor-memory columns are all there
+// are, so shared memory must not admit a fifth (the forward kernel pads its own).
 constexpr int kFwdSmem = 57344;
 constexpr int kGradSmem = GradLayout::end;
 static_assert(FwdLayout::end <= kFwdSmem, "forward tiles");
-static_assert(kGradSmem * 3 > 232448 && kGradSmem <= 232448, "two gradient CTAs per SM");
+static_assert(kGradSmem * 5 > 232448 && kGradSmem * 4 + 4 * 3072 <= 232448, "four gradient CTAs per SM");
 
 struct Ctrl {
     uint64_t mbar;
     uint32_t tmem;
     float red[4][68];   // cross-warp sums: b1 (32), b2 (32), b3 (3), loss
+    float bias[68];     // b1 (32), b2 (32), b3 (3)
 };
 
 __device__ __forceinline__ uint16_t bf16_bits(float v) {
@@ -100,20 +109,49 @@ __device__ __forceinline__ void put_row8(unsigned char* tile, int K, int row, in
     *reinterpret_cast<uint4*>(tile + tc::kmajor_offset(row, 8 * j, K)) = u;
 }
 
-// Zero the dynamic shared memory and load the weight operands (BF16).
-__device__ void load_weights(unsigned char* sm, int bytes, const float* __restrict__ P, bool transposed) {
-    for (int i = threadIdx.x * 16; i < bytes; i += blockDim.x * 16)
+// Zero bytes [from, to) of shared memory (multiples of 16).
+__device__ __forceinline__ void zero_smem(unsigned char* sm, int from, int to) {
+    for (int i = from + threadIdx.x * 16; i < to; i += kTile * 16)
         *reinterpret_cast<uint4*>(sm + i) = make_uint4(0u, 0u, 0u, 0u);
+}
+
+// Load the weight operands (BF16) into their zeroed tiles: each parameter is read
+// once, along its rows, and stored to its operand and (TRANSPOSED) the backward one.
+template <bool TRANSPOSED>
+__device__ __forceinline__ void load_weights(unsigned char* sm, const float* __restrict__ P) {
     __syncthreads();
     pdl_wait();   // the parameters may be the kernel ahead's
-    for (int i = threadIdx.x; i < kMlpH * kMlpH; i += blockDim.x) {
-        const int n = i / kMlpH, k = i % kMlpH;
-        put_bf16(sm + FwdLayout::w2, 32, n, k, P[kOffW2 + n * kMlpH + k]);
-        if (transposed) put_bf16(sm + GradLayout::w2t, 32, n, k, P[kOffW2 + k * kMlpH + n]);
-        if (k < kMlpIn) put_bf16(sm + FwdLayout::w1, 16, n, k, P[kOffW1 + n * kMlpIn + k]);
-        if (n < kMlpOut) put_bf16(sm + FwdLayout::w3, 32, n, k, P[kOffW3 + n * kMlpH + k]);
-        if (transposed && k < kMlpOut) put_bf16(sm + GradLayout::w3t, 16, n, k, P[kOffW3 + k * kMlpH + n]);
+#pragma unroll
+    for (int it = 0; it < kMlpH * kMlpH / kTile; ++it) {
+        const int i = it * kTile + threadIdx.x, n = i / kMlpH, k = i % kMlpH;
+        const float v = P[kOffW2 + i];
+        put_bf16(sm + FwdLayout::w2, 32, n, k, v);
+        if (TRANSPOSED) put_bf16(sm + GradLayout::w2t, 32, k, n, v);
     }
+    for (int i = threadIdx.x; i < kMlpH * kMlpIn; i += kTile)
+        put_bf16(sm + FwdLayout::w1, 16, i / kMlpIn, i % kMlpIn, P[kOffW1 + i]);
+    if (threadIdx.x < kMlpOut * kMlpH) {
+        const int n = threadIdx.x / kMlpH, k = threadIdx.x % kMlpH;
+        const float v = P[kOffW3 + threadIdx.x];
+        put_bf16(sm + FwdLayout::w3, 32, n, k, v);
+        if (TRANSPOSED) put_bf16(sm + GradLayout::w3t, 16, k, n, v);
+    }
+}
+
+// Sums over the warp of 32 values per lane: lane j gets the sum of value j (each
+// step keeps one half of the values and hands the other half over: 31 shuffles, a
+// butterfly of every value takes 160).
+__device__ __forceinline__ float warp_sum_transposed(float (&v)[32], int lane) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        const bool upper = lane & o;
+#pragma unroll
+        for (int j = 0; j < o; ++j) {
+            const float give = upper ? v[j] : v[j + o], keep = upper ? v[j + o] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        }
+    }
+    return v[0];
 }
 
 // Thread 0 issues the MMAs of `issue`, commits them to the mbarrier; every
@@ -140,17 +178,12 @@ __device__ void give_up(Ctrl& c, uint32_t phase) {
     tc::mbar_wait(&c.mbar, phase ^ 1u, kMaxPolls);
 }
 
-// Forward of one tile: on return h1/h2 hold this thread's activations (FP32,
-// after ReLU) and z its three logits; the BF16 operands are in shared memory.
+// Forward of one tile of the forward kernel: z its three logits.
 __device__ __forceinline__ bool tile_forward(unsigned char* sm, Ctrl& c, uint32_t& phase, uint32_t tm, int warp,
                                              int row, const float* __restrict__ P, const float (&xin)[5],
-                                             float (&h1)[32], float (&h2)[32], float (&z)[3], bool grad) {
-    {
-        const float v[8] = {xin[0], xin[1], xin[2], xin[3], xin[4], 0.f, 0.f, 0.f};
-        put_row8(sm + FwdLayout::x, 16, row, 0, v);
-        if (grad)
-            for (int k = 0; k < kMlpIn; ++k) put_bf16(sm + GradLayout::bw, kTile, 64 + k, row, xin[k]);
-    }
+                                             float (&z)[3]) {
+    const float v[8] = {xin[0], xin[1], xin[2], xin[3], xin[4], 0.f, 0.f, 0.f};
+    put_row8(sm + FwdLayout::x, 16, row, 0, v);
     if (!run_mma(c, phase, [&] {
             tc::mma_bf16(tm + 0, tc::desc_kmajor(sm + FwdLayout::x, 16, 0), tc::desc_kmajor(sm + FwdLayout::w1, 16, 0),
                          tc::idesc_bf16(kTile, 32), 0u);
@@ -159,11 +192,9 @@ __device__ __forceinline__ bool tile_forward(unsigned char* sm, Ctrl& c, uint32_
     float acc[32];
     tc::tmem_load_row<32>(tm, warp, 0, acc);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) h1[j] = fmaxf(acc[j] + P[kOffB1 + j], 0.f);
+    for (int j = 0; j < 32; ++j) acc[j] = fmaxf(acc[j] + P[kOffB1 + j], 0.f);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) put_row8(sm + FwdLayout::h1, 32, row, j, h1 + 8 * j);
-    if (grad)
-        for (int k = 0; k < kMlpH; ++k) put_bf16(sm + GradLayout::bw, kTile, k, row, h1[k]);
+    for (int j = 0; j < 4; ++j) put_row8(sm + FwdLayout::h1, 32, row, j, acc + 8 * j);
     if (!run_mma(c, phase, [&] {
             for (int s = 0; s < 2; ++s)
                 tc::mma_bf16(tm + 32, tc::desc_kmajor(sm + FwdLayout::h1, 32, s),
@@ -172,11 +203,9 @@ __device__ __forceinline__ bool tile_forward(unsigned char* sm, Ctrl& c, uint32_
         return false;
     tc::tmem_load_row<32>(tm, warp, 32, acc);
 #pragma unroll
-    for (int j = 0; j < 32; ++j) h2[j] = fmaxf(acc[j] + P[kOffB2 + j], 0.f);
+    for (int j = 0; j < 32; ++j) acc[j] = fmaxf(acc[j] + P[kOffB2 + j], 0.f);
 #pragma unroll
-    for (int j = 0; j < 4; ++j) put_row8(sm + FwdLayout::h2, 32, row, j, h2 + 8 * j);
-    if (grad)
-        for (int k = 0; k < kMlpH; ++k) put_bf16(sm + GradLayout::bw, kTile, 32 + k, row, h2[k]);
+    for (int j = 0; j < 4; ++j) put_row8(sm + FwdLayout::h2, 32, row, j, acc + 8 * j);
     if (!run_mma(c, phase, [&] {
             for (int s = 0; s < 2; ++s)
                 tc::mma_bf16(tm + 64, tc::desc_kmajor(sm + FwdLayout::h2, 32, s),
@@ -184,12 +213,7 @@ __device__ __forceinline__ bool tile_forward(unsigned char* sm, Ctrl& c, uint32_
         }))
         return false;
     float lz[8];
-    {
-        float tmp[8];
-        tc::tmem_load_row<8>(tm, warp, 64, tmp);
-#pragma unroll
-        for (int e = 0; e < 8; ++e) lz[e] = tmp[e];
-    }
+    tc::tmem_load_row<8>(tm, warp, 64, lz);
 #pragma unroll
     for (int q = 0; q < 3; ++q) z[q] = lz[q] + P[kOffB3 + q];
     return true;
@@ -210,7 +234,8 @@ __global__ void __launch_bounds__(kTile) mlp_forward_tc_kernel(const float* __re
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ Ctrl c;
     const int warp = threadIdx.x >> 5, row = threadIdx.x;
-    load_weights(sm, FwdLayout::end, P, false);
+    zero_smem(sm, 0, FwdLayout::end);
+    load_weights<false>(sm, P);
     if (threadIdx.x == 0) tc::mbar_init(&c.mbar, 1);
     if (warp == 0) tc::tmem_alloc(&c.tmem, 128);
     tc::fence_before_sync();
@@ -222,8 +247,8 @@ __global__ void __launch_bounds__(kTile) mlp_forward_tc_kernel(const float* __re
         const long long r = t0 + row;
         float xin[5];
         for (int k = 0; k < 5; ++k) xin[k] = r < B ? x[r * kMlpIn + k] : 0.f;
-        float h1[32], h2[32], z[3];
-        if (!tile_forward(sm, c, phase, tm, warp, row, P, xin, h1, h2, z, false)) {
+        float z[3];
+        if (!tile_forward(sm, c, phase, tm, warp, row, P, xin, z)) {
             give_up(c, phase);
             break;
         }
@@ -239,22 +264,64 @@ __global__ void __launch_bounds__(kTile) mlp_forward_tc_kernel(const float* __re
     if (warp == 0) tc::tmem_dealloc(tm, 128);
 }
 
-__global__ void __launch_bounds__(kTile) mlp_grad_tc_kernel(const float* __restrict__ P, const float* __restrict__ x,
-                                                            const float* __restrict__ phat,
-                                                            const float* __restrict__ target,
-                                                            const float* __restrict__ mask, long long B, float lam,
-                                                            float* __restrict__ work) {
+// Bias and ReLU of a layer's 32 accumulators (columns 0-31 of the CTA's tensor
+// memory) into columns col .. col + 31 of the activation tile; returns the bit mask of
+// the positive ones.
+__device__ __forceinline__ uint32_t relu_layer(uint32_t tm, int warp, const float* bias, unsigned char* act, int col,
+                                               int row) {
+    float h[32];
+    tc::tmem_load_row<32>(tm, warp, 0, h);
+    uint32_t on = 0;
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        h[j] = fmaxf(h[j] + bias[j], 0.f);
+        on |= h[j] > 0.f ? 1u << j : 0u;
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) put_row8(act, kCols, row, col / 8 + j, h + 8 * j);
+    return on;
+}
+
+// The same backwards: the accumulators where the activation was positive, added to
+// the bias gradient and into columns col .. of the dZ tile.
+__device__ __forceinline__ void back_layer(uint32_t tm, int warp, uint32_t on, float (&gb)[32], unsigned char* dz,
+                                           int col, int row) {
+    float d[32];
+    tc::tmem_load_row<32>(tm, warp, 0, d);
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+        d[j] = (on >> j) & 1u ? d[j] : 0.f;
+        gb[j] += d[j];
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) put_row8(dz, kCols, row, col / 8 + j, d + 8 * j);
+}
+
+__global__ void __launch_bounds__(kTile, 4) mlp_grad_tc_kernel(const float* __restrict__ P, const float* __restrict__ x,
+                                                               const float* __restrict__ phat,
+                                                               const float* __restrict__ target,
+                                                               const float* __restrict__ mask, long long B, float lam,
+                                                               float* __restrict__ work) {
     extern __shared__ __align__(1024) unsigned char sm[];
     __shared__ Ctrl c;
+    unsigned char *act = sm + GradLayout::act, *dzt = sm + GradLayout::dz;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, row = threadIdx.x;
-    load_weights(sm, GradLayout::end, P, true);
+    // weight tiles, and the columns past those a sample writes (72-79), which meet zero
+    // weights but must not be NaN
+    zero_smem(sm, 0, GradLayout::dz);
+    const float none[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    put_row8(act, kCols, row, 9, none);
+    put_row8(dzt, kCols, row, 9, none);
+    load_weights<true>(sm, P);
+    if (row < 67) c.bias[row] = P[row < 32 ? kOffB1 + row : row < 64 ? kOffB2 + row - 32 : kOffB3 + row - 64];
     if (threadIdx.x == 0) tc::mbar_init(&c.mbar, 1);
-    if (warp == 0) tc::tmem_alloc(&c.tmem, 256);
+    if (warp == 0) tc::tmem_alloc(&c.tmem, 128);
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    // columns: H1 0, H2 32, Z 64, dH2 80, dH1 112, weight gradients 144 (80 wide)
+    // columns: the layer at hand 0-31, weight gradients 32-111
     const uint32_t tm = c.tmem;
+    constexpr int kColW = 32;
     uint32_t phase = 0;
     const float invB = 1.0f / (float)B;
     float gb1[32], gb2[32], gb3[3] = {0.f, 0.f, 0.f}, lsum = 0.f;
@@ -262,20 +329,40 @@ __global__ void __launch_bounds__(kTile) mlp_grad_tc_kernel(const float* __restr
     for (int j = 0; j < 32; ++j) gb1[j] = gb2[j] = 0.f;
     bool ok = true;
     uint32_t acc_w = 0;
+    // one product of 128 samples: columns col .. of a sample tile (K-major, ksteps
+    // steps of 16) with a weight operand of K columns, N outputs
+    auto layer = [&](const unsigned char* tile, int col, const unsigned char* wt, int K, int N, int ksteps) {
+        return run_mma(c, phase, [&] {
+            for (int s = 0; s < ksteps; ++s)
+                tc::mma_bf16(tm, tc::desc_kmajor(tile + (col / 8) * 128, kCols, s), tc::desc_kmajor(wt, K, s),
+                             tc::idesc_bf16(kTile, N), (uint32_t)s);
+        });
+    };
     for (long long t0 = (long long)blockIdx.x * kTile; t0 < B && ok; t0 += (long long)gridDim.x * kTile) {
         const long long r = t0 + row;
         const bool live = r < B;
-        float xin[5];
-        for (int k = 0; k < 5; ++k) xin[k] = live ? x[r * kMlpIn + k] : 0.f;
-        float h1[32], h2[32], z[3];
-        if (!(ok = tile_forward(sm, c, phase, tm, warp, row, P, xin, h1, h2, z, true))) break;
+        float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+        float pp[3] = {0.f, 0.f, 0.f}, tt = 0.f, mk = 0.f;
+        if (live) {
+            for (int k = 0; k < kMlpIn; ++k) v[k] = x[r * kMlpIn + k];
+            for (int q = 0; q < 3; ++q) pp[q] = phat[r * 3 + q];
+            tt = target[r];
+            mk = mask[r];
+        }
+        put_row8(act, kCols, row, 8, v);
+        if (!(ok = layer(act, 64, sm + GradLayout::w1, 16, 32, 1))) break;
+        const uint32_t on1 = relu_layer(tm, warp, c.bias, act, 0, row);
+        if (!(ok = layer(act, 0, sm + GradLayout::w2, 32, 32, 2))) break;
+        const uint32_t on2 = relu_layer(tm, warp, c.bias + 32, act, 32, row);
+        if (!(ok = layer(act, 32, sm + GradLayout::w3, 32, 16, 2))) break;
+        float lz[8];
+        tc::tmem_load_row<8>(tm, warp, 0, lz);
+        const float z[3] = {lz[0] + c.bias[64], lz[1] + c.bias[65], lz[2] + c.bias[66]};
         // loss and dL/dz (zero for rows past the batch)
-        float dz[3] = {0.f, 0.f, 0.f};
+        float dz[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
         if (live) {
             float om[3];
             softmax3(z, om);
-            const float pp[3] = {phat[r * 3], phat[r * 3 + 1], phat[r * 3 + 2]};
-            const float tt = target[r], mk = mask[r];
             const float e = om[0] * pp[0] + om[1] * pp[1] + om[2] * pp[2] - tt;
             float dom[3], reg = 0.f;
 #pragma unroll
@@ -291,48 +378,17 @@ __global__ void __launch_bounds__(kTile) mlp_grad_tc_kernel(const float* __restr
         }
 #pragma unroll
         for (int q = 0; q < 3; ++q) gb3[q] += dz[q];
-        {
-            const float v[8] = {dz[0], dz[1], dz[2], 0.f, 0.f, 0.f, 0.f, 0.f};
-            put_row8(sm + GradLayout::dz3, 16, row, 0, v);
-            for (int q = 0; q < 3; ++q) put_bf16(sm + GradLayout::aw, kTile, 64 + q, row, dz[q]);
-        }
-        // dH2 = dZ W3, dZ2 = dH2 * (H2 > 0)
-        if (!(ok = run_mma(c, phase, [&] {
-                  tc::mma_bf16(tm + 80, tc::desc_kmajor(sm + GradLayout::dz3, 16, 0),
-                               tc::desc_kmajor(sm + GradLayout::w3t, 16, 0), tc::idesc_bf16(kTile, 32), 0u);
-              })))
-            break;
-        float d[32];
-        tc::tmem_load_row<32>(tm, warp, 80, d);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            d[j] = h2[j] > 0.f ? d[j] : 0.f;
-            gb2[j] += d[j];
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) put_row8(sm + GradLayout::dz2, 32, row, j, d + 8 * j);
-        for (int k = 0; k < kMlpH; ++k) put_bf16(sm + GradLayout::aw, kTile, k, row, d[k]);
-        // dH1 = dZ2 W2, dZ1 = dH1 * (H1 > 0)
-        if (!(ok = run_mma(c, phase, [&] {
-                  for (int s = 0; s < 2; ++s)
-                      tc::mma_bf16(tm + 112, tc::desc_kmajor(sm + GradLayout::dz2, 32, s),
-                                   tc::desc_kmajor(sm + GradLayout::w2t, 32, s), tc::idesc_bf16(kTile, 32),
-                                   (uint32_t)s);
-              })))
-            break;
-        tc::tmem_load_row<32>(tm, warp, 112, d);
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-            d[j] = h1[j] > 0.f ? d[j] : 0.f;
-            gb1[j] += d[j];
-        }
-        for (int k = 0; k < kMlpH; ++k) put_bf16(sm + GradLayout::aw, kTile, 32 + k, row, d[k]);
+        put_row8(dzt, kCols, row, 8, dz);
+        // dH2 = dZ W3, dZ2 = dH2 * (H2 > 0); dH1 = dZ2 W2, dZ1 = dH1 * (H1 > 0)
+        if (!(ok = layer(dzt, 64, sm + GradLayout::w3t, 16, 32, 1))) break;
+        back_layer(tm, warp, on2, gb2, dzt, 0, row);
+        if (!(ok = layer(dzt, 0, sm + GradLayout::w2t, 32, 32, 2))) break;
+        back_layer(tm, warp, on1, gb1, dzt, 32, row);
         // weight gradients: accumulate over the batch (eight K steps of 16 samples)
         if (!(ok = run_mma(c, phase, [&] {
                   for (int s = 0; s < kTile / 16; ++s)
-                      tc::mma_bf16(tm + 144, tc::desc_kmajor(sm + GradLayout::aw, kTile, s),
-                                   tc::desc_kmajor(sm + GradLayout::bw, kTile, s), tc::idesc_bf16(kTile, kBWN),
-                                   acc_w | (uint32_t)s);
+                      tc::mma_bf16(tm + kColW, tc::desc_mnmajor(dzt, kCols, s), tc::desc_mnmajor(act, kCols, s),
+                                   tc::idesc_bf16_mn(kTile, kCols), acc_w | (uint32_t)s);
               })))
             break;
         acc_w = 1u;
@@ -344,7 +400,7 @@ __global__ void __launch_bounds__(kTile) mlp_grad_tc_kernel(const float* __restr
         // weight gradients: warp 0 rows dW2, warp 1 rows dW1, warp 2 lanes 0..2 rows dW3
         if (acc_w && warp < 3) {
             float dw[32];
-            tc::tmem_load_row<32>(tm, warp, 144 + (warp == 0 ? 0 : warp == 1 ? 64 : 32), dw);
+            tc::tmem_load_row<32>(tm, warp, kColW + (warp == 0 ? 0 : warp == 1 ? 64 : 32), dw);
             if (warp == 0) {
                 for (int k = 0; k < kMlpH; ++k) out[kOffW2 + lane * kMlpH + k] = dw[k];
             } else if (warp == 1) {
@@ -357,22 +413,15 @@ __global__ void __launch_bounds__(kTile) mlp_grad_tc_kernel(const float* __restr
                 if (!(i >= kOffB1 && i < kOffW2) && !(i >= kOffB2 && i < kOffW3)) out[i] = 0.f;
         }
         // bias gradients and loss: warp sums, then across the four warps
+        c.red[warp][lane] = warp_sum_transposed(gb1, lane);
+        c.red[warp][32 + lane] = warp_sum_transposed(gb2, lane);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {
-#pragma unroll
-            for (int j = 0; j < 32; ++j) {
-                gb1[j] += __shfl_xor_sync(0xffffffffu, gb1[j], o);
-                gb2[j] += __shfl_xor_sync(0xffffffffu, gb2[j], o);
-            }
 #pragma unroll
             for (int q = 0; q < 3; ++q) gb3[q] += __shfl_xor_sync(0xffffffffu, gb3[q], o);
             lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
         }
         if (lane == 0) {
-            for (int j = 0; j < 32; ++j) {
-                c.red[warp][j] = gb1[j];
-                c.red[warp][32 + j] = gb2[j];
-            }
             for (int q = 0; q < 3; ++q) c.red[warp][64 + q] = gb3[q];
             c.red[warp][67] = lsum;
         }
@@ -387,7 +436,7 @@ __global__ void __launch_bounds__(kTile) mlp_grad_tc_kernel(const float* __restr
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
-    if (warp == 0) tc::tmem_dealloc(tm, 256);
+    if (warp == 0) tc::tmem_dealloc(tm, 128);
 }
 
 unsigned grid_for(long long B, int per_sm) {
@@ -420,8 +469,8 @@ mfc_status mfc_mlp_grad(const float* params, const float* x, const float* phat, 
     if (cudaFuncSetAttribute(mlp_grad_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGradSmem) !=
         cudaSuccess)
         return MFC_ERR_CUDA;
-    const unsigned blocks = grid_for(batch, 2);
-    static_assert(2LL * 152 * kTcStride <= MFC_MLP_WORK_FLOATS, "workspace holds every CTA's partial");
+    const unsigned blocks = grid_for(batch, 4);
+    static_assert(4LL * 152 * kTcStride <= MFC_MLP_WORK_FLOATS, "workspace holds every CTA's partial");
     if (launch_pdl(mlp_grad_tc_kernel, blocks, kTile, kGradSmem, s, params, x, phat, target, mask, batch, lam, work) !=
         cudaSuccess)
         return MFC_ERR_CUDA;

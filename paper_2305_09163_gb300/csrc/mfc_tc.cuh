@@ -36,12 +36,27 @@ __device__ __forceinline__ uint64_t desc_kmajor(const void* tile, int K, int kst
            ((uint64_t)((uint32_t)(16 * K) >> 4) << 32) | (1ull << 46);
 }
 
+// Descriptor of the same tile read across (MN-major, unswizzled): its columns are
+// the M or N index and its rows the K index, so a tile [sample][feature] serves as
+// the transposed operand of a contraction over the samples without being copied.
+// A core matrix is then 8 K rows x 16 bytes of M or N; groups of 8 rows (K) are
+// 16 K-tile-columns bytes apart (leading-dimension offset), groups of 8 columns
+// (M, N) 128 bytes (stride-dimension offset).  kstep: steps of 16 rows.
+__device__ __forceinline__ uint64_t desc_mnmajor(const void* tile, int K, int kstep) {
+    const uint32_t a = smem_u32(tile) + (uint32_t)(kstep * 32 * K);
+    return (uint64_t)((a & 0x3FFFFu) >> 4) | ((uint64_t)((uint32_t)(16 * K) >> 4) << 16) |
+           ((uint64_t)(128u >> 4) << 32) | (1ull << 46);
+}
+
 // Instruction descriptor of kind::f16 with BF16 A and B, FP32 D, both K-major,
 // dense: D format (bits 4-5) = 1, A format (7-9) = 1, B format (10-12) = 1,
 // N >> 3 (17-22), M >> 4 (24-28).
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
+
+// The same with A and B MN-major (bits 15 and 16).
+__host__ __device__ constexpr uint32_t idesc_bf16_mn(int M, int N) { return idesc_bf16(M, N) | (1u << 15) | (1u << 16); }
 
 // TMEM allocation of ncols columns (a power of two >= 32) by one whole warp;
 // the base address is written to *slot in shared memory.
@@ -113,27 +128,26 @@ __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
                  : "memory");
 }
 
-__device__ __forceinline__ void tmem_wait(uint32_t (&r)[8]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
-                 :
-                 : "memory");
+// All loads of N columns are issued before the one wait.
+template <int N>
+__device__ __forceinline__ void tmem_wait(uint32_t (&r)[N]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int j = 0; j < N; ++j) asm volatile("" : "+r"(r[j])::"memory");   // no use moves above the wait
 }
 
-// n (a multiple of 8) FP32 columns starting at column col of this thread's lane
+// N (a multiple of 8) FP32 columns starting at column col of this thread's lane
 // (warp w of the warpgroup reads lanes 32 w .. 32 w + 31).
 template <int N>
 __device__ __forceinline__ void tmem_load_row(uint32_t tmem_base, int warp, int col, float (&out)[N]) {
     static_assert(N % 8 == 0, "columns in groups of eight");
     const uint32_t t = tmem_base + ((uint32_t)(32 * warp) << 16) + (uint32_t)col;
+    uint32_t r[N];
 #pragma unroll
-    for (int j = 0; j < N / 8; ++j) {
-        uint32_t r[8];
-        tmem_ld8(t + 8 * j, r);
-        tmem_wait(r);
+    for (int j = 0; j < N / 8; ++j) tmem_ld8(t + 8 * j, *reinterpret_cast<uint32_t(*)[8]>(&r[8 * j]));
+    tmem_wait(r);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) out[8 * j + e] = __uint_as_float(r[e]);
-    }
+    for (int e = 0; e < N; ++e) out[e] = __uint_as_float(r[e]);
 }
 
 }  // namespace tc
