@@ -391,7 +391,6 @@ mfc_status run_sweeps(mfc_ctx* c, double* out, const RkStage* rk, void* w_next =
             a.c0 = rk->c0;
             a.c1 = rk->c1;
             a.dt = rk->dt;
-            a.c1dtd = df_split(rk->c1 * rk->dt);
             a.w_next = w_next;
             a.rate_max = rate ? c->d_rate : nullptr;
             a.bad = rate ? bad_count(c) : nullptr;

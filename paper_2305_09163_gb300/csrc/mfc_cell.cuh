@@ -662,11 +662,14 @@ __device__ __forceinline__ double finish_cell_rates_df(const SweepArgs& a, long 
         for (int v = 0; v < NQ; ++v) R[v * nc + idx] = df_add_fast(pR[v * sRv], out[v]);
     } else if (a.mode == 2) {
         double qn[NQ];
-        // c1 qs + c0 q0 + c1 dt R, the last product in float-float before it is
-        // widened: one FP64 instruction per value fewer
+        // c1 (qs + dt R), the product skipped when c1 = 1, + c0 q0.  (c1 dt R in
+        // float-float before it is widened saves an FP64 instruction per value but
+        // raised the error of a step against 64 bits by 2-10%.)
+        const bool unit = a.c1 == 1.0;
 #pragma unroll
         for (int v = 0; v < NQ; ++v) {
-            double o = fma(a.c1, qsv(v), df_to_double(df_prod(total(v), a.c1dtd)));
+            double o = fma(a.dt, df_to_double(total(v)), qsv(v));
+            if (!unit) o *= a.c1;
             if (a.c0 != 0.0) o = fma(a.c0, q0v(v), o);
             qn[v] = o;
             a.qout[v * nc + idx] = o;

@@ -115,7 +115,7 @@ struct SweepArgs {
     float epsf;
     float inv_dxf[3];
     EosDf ed;               // FP64 kernels: e, eps * 3/4, eps and g.inv_dx in float-float
-    df eps34d, epsd, inv_dxd[3], c1dtd;   // c1dtd: c1 dt of an RK stage
+    df eps34d, epsd, inv_dxd[3];
     df kgamd[3], kpinfd[3];     // kgam, kpinf in float-float
 };
 
@@ -153,7 +153,6 @@ inline void sweep_set_constants(SweepArgs& a) {
     }
     a.eps34d = df_split(0.75 * a.eps);
     a.epsd = df_split(a.eps);
-    a.c1dtd = df_split(a.c1 * a.dt);
     for (int d = 0; d < 3; ++d) a.inv_dxd[d] = df_split(a.g.inv_dx[d]);
     for (int k = 0; k < 3; ++k) {
         a.kgamd[k] = df_split(a.kgam[k]);
