@@ -175,8 +175,8 @@ __global__ void __launch_bounds__(128) sweep_kernel(const SweepArgs a) {
 // true).
 // ---------------------------------------------------------------------------
 template <typename Real, int NF, int NDIM, int ORDER, bool NONUNIF, bool SIX, bool VALUE_MAJOR>
-__device__ __forceinline__ void dfs_edges(const SweepArgs& a, int dir, int c, int q, double vc, const df (&D)[4],
-                                          df& eR, df& eL) {
+__device__ __forceinline__ void dfs_edges(const SweepArgs& a, int dir, int c, int q, double vc, df cc,
+                                          const df (&D)[4], df& eR, df& eL) {
     df2 I;
     if constexpr (NONUNIF) {
         const GridCol<VALUE_MAJOR> grow(a.grid[dir], a.grid_stride[dir], c);
@@ -190,7 +190,6 @@ __device__ __forceinline__ void dfs_edges(const SweepArgs& a, int dir, int c, in
         eL = df_pack(vc + df_to_double(df2_x(I)));
         eR = df_pack(vc + df_to_double(df2_y(I)));
     } else {
-        const df cc = df_from_double_rn(vc);
         const df2 E = df2_add_fast(df2_make(cc, cc), I);
         eL = df2_x(E);
         eR = df2_y(E);
@@ -382,7 +381,8 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
                 const df Dq[4] = {df_from_double(v[1] - v[0]), df_from_double(v[2] - v[1]), df_from_double(v[3] - v[2]),
                                   df_from_double(v[4] - v[3])};
                 df er, el;
-                dfs_edges<Real, NF, NDIM, ORDER, NONUNIF, SIX, true>(a, 0, c, q, v[2], Dq, er, el);
+                dfs_edges<Real, NF, NDIM, ORDER, NONUNIF, SIX, true>(a, 0, c, q, v[2], df_from_double_rn(v[2]), Dq, er,
+                                                                     el);
                 dsh_eL[q][pos] = el;
                 dsh_eR[q][t] = er;
             }
@@ -613,7 +613,19 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
     // ROLL (FP64): one copy of the reconstruction looped over the variables
     // (stencils from the ring, edges to shared memory); see the x stream body.
     constexpr bool ROLL = sizeof(Real) == 8 && !LEARNED;
+    // TRI (FP64 five-equation): the rows are kept in three FP32 parts, split once
+    // where they arrive, and the stencil's differences are taken from the parts: no
+    // FP64 subtraction (28 per cell, a third to a half of the sweep's FP64
+    // instructions) and one split per value instead of five.  256^3: y 2496 -> 2419,
+    // z 3449 -> 3042 us; 100x90x77: y 124.0 -> 122.5, z 140.9 -> 138.5.  Where one
+    // wave of blocks holds the whole grid the chain of each chunk counts instead of
+    // the FP64 pipe: 48x41x33 y 26.1 -> 24.5, z 26.8 -> 29.8.  Not the six-equation
+    // model (its interior edge values are FP64 sums) nor the x sweep, whose rows stay
+    // in value-major FP64 for its staged loads
+    constexpr bool TRI = sizeof(Real) == 8 && !LEARNED && !SIX;
     __shared__ Real ring[RING][NS][32];
+    __shared__ float ring_lo[TRI ? RING : 1][TRI ? NS : 1][32];
+    df(*ring_hm)[NS][32] = reinterpret_cast<df(*)[NS][32]>(ring);   // TRI: (hi, mid)
     __shared__ Real sh_eL[NS][ER][32];
     __shared__ Real sh_eR[(ROLL || LEARNED) ? NS : 1][kRowsPerChunk][32];
     // DFS: edge values kept in float-float into the Riemann solver (x stream body)
@@ -670,6 +682,18 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
     };
     auto slot = [](int i) { return ((i % RING) + RING) % RING; };
     auto eslot = [](int i) { return (i + 2 * ER) % ER; };   // i >= -2
+    auto store_row = [&](int i, const Real* v) {
+#pragma unroll
+        for (int q = 0; q < NS; ++q) {
+            if constexpr (TRI) {
+                const tf x = tf_from_double(v[q]);
+                ring_hm[slot(i)][q][lane] = {x.hi, x.mid};
+                ring_lo[slot(i)][q][lane] = x.lo;
+            } else {
+                ring[slot(i)][q][lane] = v[q];
+            }
+        }
+    };
     // prologue: rows s0-3 .. s0+4 (cells base-2 .. base+5 of the first chunk)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
@@ -677,8 +701,7 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
         if (i <= s1 + 2) {
             Real v[NS];
             load(i, v);
-#pragma unroll
-            for (int q = 0; q < NS; ++q) ring[slot(i)][q][lane] = v[q];
+            store_row(i, v);
         }
     }
     __syncthreads();
@@ -734,21 +757,46 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
                 }
             } else if constexpr (ROLL) {
                 const int s0r = slot(c - 2), s1r = slot(c - 1), s2r = slot(c), s3r = slot(c + 1), s4r = slot(c + 2);
-#pragma unroll 1
-                for (int q = 0; q < NS; ++q) {
-                    const Real v0 = ring[s0r][q][lane], v1 = ring[s1r][q][lane], vc = ring[s2r][q][lane];
-                    const Real v3 = ring[s3r][q][lane], v4 = ring[s4r][q][lane];
-                    const df Dq[4] = {df_from_double(v1 - v0), df_from_double(vc - v1), df_from_double(v3 - vc),
-                                      df_from_double(v4 - v3)};
-                    df er, el;
-                    dfs_edges<Real, NF, NDIM, ORDER, NONUNIF, SIX, false>(a, DIR, c, q, vc, Dq, er, el);
-                    dsh_eL[q][eslot(c)][lane] = el;
-                    dsh_eR[q][row][lane] = er;
-                }
+                if constexpr (TRI) {
+                    // the finished cell's values for the source terms (c - 1 >= s0: no ghost)
+                    if (fin) {
+                        const Real* p = w + basei + (unsigned)(c - 1) * sd;
 #pragma unroll
-                for (int q = 0; q < NS; ++q) {
-                    cell[q] = ring[s2r][q][lane];
-                    cm1[q] = ring[s1r][q][lane];
+                        for (int q = 0; q < NS; ++q)
+                            if (q >= Lay::IA || (q == Lay::IE && a.kapila)) cm1[q] = __ldg(p + q * nc);
+                    }
+#pragma unroll 1
+                    for (int q = 0; q < NS; ++q) {
+                        auto part = [&](int r) -> tf {
+                            const df h = ring_hm[r][q][lane];
+                            return {h.hi, h.lo, ring_lo[r][q][lane]};
+                        };
+                        const tf x0 = part(s0r), x1 = part(s1r), x2 = part(s2r), x3 = part(s3r), x4 = part(s4r);
+                        const df Dq[4] = {tf_diff(x1, x0), tf_diff(x2, x1), tf_diff(x3, x2), tf_diff(x4, x3)};
+                        df er, el;
+                        dfs_edges<Real, NF, NDIM, ORDER, NONUNIF, SIX, false>(
+                            a, DIR, c, q, 0.0, {x2.hi, __fadd_rn(x2.mid, x2.lo)}, Dq, er, el);
+                        dsh_eL[q][eslot(c)][lane] = el;
+                        dsh_eR[q][row][lane] = er;
+                    }
+                } else {
+#pragma unroll 1
+                    for (int q = 0; q < NS; ++q) {
+                        const Real v0 = ring[s0r][q][lane], v1 = ring[s1r][q][lane], vc = ring[s2r][q][lane];
+                        const Real v3 = ring[s3r][q][lane], v4 = ring[s4r][q][lane];
+                        const df Dq[4] = {df_from_double(v1 - v0), df_from_double(vc - v1), df_from_double(v3 - vc),
+                                          df_from_double(v4 - v3)};
+                        df er, el;
+                        dfs_edges<Real, NF, NDIM, ORDER, NONUNIF, SIX, false>(a, DIR, c, q, vc, df_from_double_rn(vc),
+                                                                              Dq, er, el);
+                        dsh_eL[q][eslot(c)][lane] = el;
+                        dsh_eR[q][row][lane] = er;
+                    }
+#pragma unroll
+                    for (int q = 0; q < NS; ++q) {
+                        cell[q] = ring[s2r][q][lane];
+                        cm1[q] = ring[s1r][q][lane];
+                    }
                 }
             } else {
                 Real Dv[NS][4];
@@ -781,10 +829,7 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
         }
         __syncthreads();
         // rows base-2 .. base+1 are no longer needed: the prefetched rows replace them
-        if (pf) {
-#pragma unroll
-            for (int q = 0; q < NS; ++q) ring[slot(inext)][q][lane] = nxt[q];
-        }
+        if (pf) store_row(inext, nxt);
         Real F[NQ], ut = 0;
         [[maybe_unused]] df Fd[DFS ? NQ : 1], utd = {0.f, 0.f};
         const bool has_face = live && c >= s0;
@@ -796,7 +841,13 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
                 lftd[q] = dsh_eL[q][eslot(c - 1)][lane];
                 erd[q] = dsh_eR[q][row][lane];
             }
-            auto cells = [&](int v, int side) -> double { return side ? cell[v] : cm1[v]; };
+            auto cells = [&](int v, int side) -> double {
+                if constexpr (!TRI) return side ? cell[v] : cm1[v];
+                bool flip = false;
+                const int m = ghost_map(c - 1 + side, nd, bclo, bchi, &flip);
+                const double x = __ldg(w + v * nc + basei + (unsigned)m * sd);
+                return v == IM + DIR && flip ? -x : x;
+            };
             face_flux_df<NF, NDIM, DIR, SIX>(a, lftd, erd, cells, Fd, utd);
 #pragma unroll
             for (int q = 0; q < NQ; ++q) dsh_F[q][eslot(c)][lane] = Fd[q];
