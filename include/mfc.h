@@ -56,13 +56,14 @@ typedef enum {
 } mfc_bc;
 
 /* Arithmetic of the reconstruction and Riemann solver:
- *   MFC_FP64    float64 state, primitive recovery, stencil differences, edge
- *               sums, mixture rules, fluxes, divergence and Runge-Kutta
- *               update; the WENO nonlinear weights and the HLLC solver are
- *               evaluated in float-float arithmetic (a value is the unevaluated
+ *   MFC_FP64    float64 state, primitive recovery, source coefficients and
+ *               Runge-Kutta update; stencil differences are exact differences
+ *               of the float64 primitives; reconstruction, mixture rules, HLLC
+ *               solver, divergence and the sum over directions are evaluated
+ *               in float-float arithmetic (a value is the unevaluated
  *               sum of two float32 numbers, about 48 significant bits) with the
- *               float32 exponent range, and their results are widened back to
- *               float64.  The right-hand side matches a plain float64
+ *               float32 exponent range, and the right-hand side is widened back
+ *               to float64.  It matches a plain float64
  *               evaluation to 1e-11 relative to each component's flux scale.
  *               Supported range (SI units): every primitive value, stencil
  *               difference and pressure jump below 1e18 in magnitude (the

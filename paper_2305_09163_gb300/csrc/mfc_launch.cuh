@@ -85,10 +85,9 @@ cudaError_t launch_yz_stream(Kernel kernel, unsigned blocks, SweepArgs a, int nq
 // SIX: the six-equation model (stream kernels, WENO5, uniform grids).
 template <typename Real, int NF, bool LEARNED = false, int ORDER = 5, bool NONUNIF = false, bool SIX = false>
 cudaError_t launch_sweep(SweepArgs a, int ndim, int dir, cudaStream_t s) {
-    // FP64 x sweeps bounded to 4 CTAs per SM (128 registers, small spills):
-    // faster for the stretched-grid (83.7 -> 71.1 ms per step at 256^3),
-    // six-equation (83.4 -> 80.7) and WENO3 (42.1 -> 41.5) variants, slower
-    // for the uniform WENO5 ones (61.0 -> 63.8, Kapila 65.3 -> 67.2)
+    // FP64 x sweeps bounded to 4 CTAs per SM (128 registers): the stretched-grid,
+    // six-equation and WENO3 variants, which take more when left unbounded; the
+    // uniform WENO5 one fits 4 CTAs without a bound
     constexpr bool kBoundFp64 = NONUNIF || SIX || ORDER == 3;
     if (dir == 0) {
         const long long total = (long long)(a.g.n[0] + 2) * (a.g.ncell / a.g.n[0]);
