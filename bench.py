@@ -86,22 +86,22 @@ SCHEDULERS = 152 * 4
 # Warp instructions per cell of the FP64 WENO5 sweeps (x, y, z; 3D, two
 # fluids, smsp__inst_executed.sum / cells of one ncu capture).  Re-measured
 # whenever the FP64 sweeps change: NCU_FP64_SWEEPS says which capture.
-FP64_SWEEP_WARP_INST_PER_CELL = (173.4, 176.9, 187.1)
+FP64_SWEEP_WARP_INST_PER_CELL = (130.5, 130.4, 146.7)
 # From the same capture: FP64-pipe and FP32 (fma) pipe activity of the sweeps
 # (mean over x, y, z) and DRAM bytes per cell per launch (the z sweep of an RK
 # stage also writes the next stage's primitives).
-FP64_SWEEP_PIPE_FP64 = 0.404
-FP64_SWEEP_PIPE_FMA = 0.588
-FP64_SWEEP_DRAM_BYTES_PER_CELL = (101.7 + 158.1 + 334.9) / 3.0
+FP64_SWEEP_PIPE_FP64 = 0.279
+FP64_SWEEP_PIPE_FMA = 0.642
+FP64_SWEEP_DRAM_BYTES_PER_CELL = (101.7 + 156.8 + 331.1) / 3.0
 NCU_FP64_SWEEPS = "profiles/sweep_fp64_shock_bubble_160.md"
 # The same count for the other FP64 forms (x, y, z; 160^3 shock-bubble, RK
 # stage 2; profiles/sweep_fp64_forms_shock_bubble_160.md).
 FP64_SWEEP_WARP_INST_PER_CELL_FORM = {
-    "fp64_weno3": (114.7, 117.0, 127.6),
-    "fp64_kapila": (187.2, 189.8, 200.1),
-    "fp64_stretched": (221.4, 206.6, 217.6),
-    "fp64_cbc": (174.1, 177.2, 187.5),
-    "fp64_six": (188.6, 191.7, 261.2),
+    "fp64_weno3": (86.5, 90.3, 106.6),
+    "fp64_kapila": (142.5, 141.8, 158.0),
+    "fp64_stretched": (169.1, 160.8, 177.5),
+    "fp64_cbc": (132.3, 130.9, 147.1),
+    "fp64_six": (145.6, 149.1, 161.6),
 }
 NCU_FP64_FORMS = "profiles/sweep_fp64_forms_shock_bubble_160.md"
 # Nominal FP32 peak: 152 SMs x 128 FMA/clk x 2 FLOP x 2.07 GHz
@@ -752,7 +752,7 @@ def main():
                    "rhs_per_step": 3, "cfl": CFL, "develop_steps": args.develop,
                    "parallelism": "replicas" if ws > 1 else "single-gpu",
                    "l2": "inputs larger than L2 (state %.2f GB per array)" % (cells * ns * 8 / 1e9),
-                   "arithmetic": "FP64 state, primitives, differences, fluxes, RK; WENO weights and HLLC in "
+                   "arithmetic": "FP64 state, primitives, sources, RK; reconstruction, HLLC, fluxes and R in "
                                  "float-float (~48 bits, FP32 exponent range); parity <= 1e-11 vs the FP64 oracle"},
         "cell_updates_per_s": ws * cells / (ms * 1e-3),
         "roofline": _sweep_roofline_fp64(fp, cells, ns, "weno5", wl.nf, fp["clocks"]) if head == "fp64" else None,
@@ -777,7 +777,7 @@ def main():
             entry["roofline"]["note"] = ("instruction count per cell of this form's sweeps (ncu); FLOPs of the "
                                          "oracle's %s formulation%s"
                                          % (work, "; the per-cell tables of the stretched grid and the "
-                                            "six-equation rows and relaxation add work" if variant in
+                                            "six-equation rows add work" if variant in
                                             ("stretched", "six") else ""))
         else:
             entry["roofline"] = _sweep_roofline_hbm(r, cells, neq, ns, work, wl.nf, peaks,

@@ -259,7 +259,7 @@ __device__ __forceinline__ void relax6(const RelaxConst& c, const EosConst& e, d
 // in one pass over it: the relaxed fractions and phase energies go back to q,
 // the primitives to w.  In the epilogue of the last sweep the relaxation held up
 // the sweep's barriers with 16 warps per SM (112x104x96 FP64: z sweep 700 us, then
-// 44 us of recovery or 100 us of CFL pass; now 387 us and 137 or 173 us).
+// 44 us of recovery or 100 us of CFL pass; now 387 us and 137 or 151 us).
 template <typename Real, int NF, int NDIM, bool RATE>
 __global__ void __launch_bounds__(256) relax_prims_kernel(const PrimArgs a, const RelaxConst c) {
     using Lay = Layout<NF, NDIM, true>;

@@ -924,7 +924,8 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
 
 // The mixed form's y/z stream kernel on non-uniform grids, bounded to 5 CTAs per
 // SM (96 registers, no spills; three fluids 4 and 128): left alone the z sweep took
-// 126 registers and ran 4 (256^3 z sweep 1.35 -> 1.11 ms).  No staging (it took the kernel from 96 to 123 registers).
+// 126 registers and ran 4 (256^3 z sweep 1.35 -> 1.11 ms).  No staging (it took the
+// kernel from 96 to 123 registers).
 template <int NF, int NDIM, int DIR>
 __global__ void __launch_bounds__(32 * kRowsPerChunk, NF <= 2 ? 5 : 4) sweep_yz_stream_f32_nu_kernel(const SweepArgs a) {
     sweep_yz_stream_body<float, NF, NDIM, DIR, false, 5, true>(a);
