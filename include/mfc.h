@@ -57,8 +57,9 @@ typedef enum {
 
 /* Arithmetic of the reconstruction and Riemann solver:
  *   MFC_FP64    float64 state, primitive recovery, source coefficients and
- *               Runge-Kutta update; stencil differences are exact differences
- *               of the float64 primitives; reconstruction, mixture rules, HLLC
+ *               Runge-Kutta update; stencil differences are those of the
+ *               float64 primitives, rounded once to the ~48 bits below;
+ *               reconstruction, mixture rules, HLLC
  *               solver, divergence and the sum over directions are evaluated
  *               in float-float arithmetic (a value is the unevaluated
  *               sum of two float32 numbers, about 48 significant bits) with the
