@@ -70,9 +70,12 @@ typedef enum {
  *               difference and pressure jump below 1e18 in magnitude (the
  *               smoothness indicators square the differences in float32
  *               range), every product of three state values such as
- *               (rho E + p) u below 1e37; a magnitude below 2^-126 (1.2e-38)
+ *               (rho E + p) u below 1e37, for cells of any size (the sums over
+ *               directions are scaled by a power of two near the smallest dx);
+ *               a magnitude below 2^-126 (1.2e-38)
  *               inside these solvers counts as zero, an absolute error far
- *               below any flux scale;
+ *               below any flux scale.  Fluxes above that range give infinities
+ *               or NaNs in the right-hand side, which the CFL check reports;
  *   MFC_MIXED   WENO5 and HLLC in float32; pressure recovery from total energy
  *               and the Runge-Kutta accumulation stay float64;
  *   MFC_LEARNED as MFC_MIXED, with WENO5 nonlinear weights from a small MLP

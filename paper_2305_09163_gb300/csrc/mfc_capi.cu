@@ -58,6 +58,7 @@ struct mfc_ctx {
     int six = 0;              // model 2: six-equation model with pressure relaxation
     int nw = 3;               // primitive rows (2N + d); ns = state rows (+N for the six-equation model)
     float* grid[3] = {nullptr, nullptr, nullptr};   // non-uniform directions: WENO5 rows (mfc_grid.cu)
+    double grid_max_inv_dx[3] = {0, 0, 0};          // and the reciprocal of their narrowest cell
     void* cbc_rates = nullptr;    // characteristic boundaries: rates of the boundary cells
     size_t cbc_bytes = 0;
 
@@ -305,7 +306,9 @@ SweepArgs base_sweep(const mfc_ctx* c) {
         a.kgam[k] = k < c->nf ? c->gamma[k] : 1.0;
         a.kpinf[k] = k < c->nf ? c->pi_inf[k] : 0.0;
     }
-    sweep_set_constants(a);
+    double max_inv_dx = 0.0;
+    for (int d = 0; d < c->ndim; ++d) max_inv_dx = fmax(max_inv_dx, c->grid[d] ? c->grid_max_inv_dx[d] : c->g.inv_dx[d]);
+    sweep_set_constants(a, max_inv_dx);
     return a;
 }
 
@@ -633,6 +636,9 @@ mfc_status mfc_set_grid(mfc_ctx* c, int dir, const double* faces, int nfaces) {
     MFC_CUDA(c, cudaMemcpyAsync(c->grid[dir], tab.data(), tab.size() * sizeof(float), cudaMemcpyHostToDevice,
                                 c->stream));
     MFC_CUDA(c, cudaStreamSynchronize(c->stream));
+    double least = faces[1] - faces[0];
+    for (int i = 1; i < c->n[dir]; ++i) least = fmin(least, faces[i + 1] - faces[i]);
+    c->grid_max_inv_dx[dir] = 1.0 / least;
     c->rate_valid = false;   // the CFL rate depends on the widths
     return MFC_OK;
 }

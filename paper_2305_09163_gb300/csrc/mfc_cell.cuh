@@ -496,7 +496,8 @@ __device__ __forceinline__ void publish_rate(const SweepArgs& a, const RateAcc& 
 // a separate recovery pass over q) and, with a.rate_max, its CFL rate is
 // returned for the caller's RateAcc (-1: non-physical); otherwise 0.
 //
-// The FP64 path keeps the accumulator R in float-float (the same 8 bytes): its
+// The FP64 path keeps the accumulator R in float-float (the same 8 bytes), scaled
+// by a power of two (SweepArgs::r_exp): its
 // sweeps' contributions are float-float differences good to ~2^-47 of the fluxes,
 // so FP64 sums of them only cost a widening and two FP64 additions per value and
 // sweep (256^3 x / y / z sweep 2.78 / 2.67 / 3.74 -> 2.69 / 2.59 / 3.64 ms).
@@ -609,6 +610,16 @@ __device__ __forceinline__ double finish_cell_rates(const SweepArgs& a, long lon
     return 0.0;
 }
 
+// A rate formed in FP64 as the accumulator holds it: scaled, float-float; NaN where
+// that is not finite or beyond the FP32 range.
+__device__ __forceinline__ df df_rate(const SweepArgs& a, double r) {
+    r *= df_widen(a.r_scale);
+    const df x = df_from_double_rn(r);
+    return ((unsigned)__double2hiint(r) & 0x7FF00000u) < (1023u + 127u) << 20 ? x : df{NAN, 0.f};
+}
+
+// The rates in out and the face-velocity divergence du come in scaled by
+// a.r_scale.
 template <int NF, int NDIM, int DIR, bool SIX = false>
 __device__ __forceinline__ double finish_cell_rates_df(const SweepArgs& a, long long idx, df* out, df du,
                                                        const double* cell, double inv_dx, int b, long long sd,
@@ -637,7 +648,7 @@ __device__ __forceinline__ double finish_cell_rates_df(const SweepArgs& a, long 
         double cb[NS];
         if (cbc_stored_rate<double, NF, NDIM, DIR>(a, idx, inv_dx, b, sd, cb)) {
 #pragma unroll
-            for (int v = 0; v < NS; ++v) out[v] = df_from_double(cb[v]);
+            for (int v = 0; v < NS; ++v) out[v] = df_rate(a, cb[v]);
         }
     }
     const long long nc = a.g.ncell;
@@ -668,7 +679,7 @@ __device__ __forceinline__ double finish_cell_rates_df(const SweepArgs& a, long 
         const bool unit = a.c1 == 1.0;
 #pragma unroll
         for (int v = 0; v < NQ; ++v) {
-            double o = fma(a.dt, df_to_double(total(v)), qsv(v));
+            double o = fma(a.dt, df_to_double_scaled(total(v), a.r_exp), qsv(v));
             if (!unit) o *= a.c1;
             if (a.c0 != 0.0) o = fma(a.c0, q0v(v), o);
             qn[v] = o;
@@ -686,7 +697,7 @@ __device__ __forceinline__ double finish_cell_rates_df(const SweepArgs& a, long 
         }
     } else {
 #pragma unroll
-        for (int v = 0; v < NQ; ++v) a.out[v * nc + idx] = df_to_double(total(v));
+        for (int v = 0; v < NQ; ++v) a.out[v * nc + idx] = df_to_double_scaled(total(v), a.r_exp);
     }
     return 0.0;
 }
@@ -703,9 +714,9 @@ __device__ __forceinline__ double finish_cell(const SweepArgs& a, long long idx,
         for (int v = 0; v < NQ; ++v) {
             double o = (Fm[v] - Fp[v]) * inv_dx;
             if (v >= IA && v < IA + NF - 1) o = fma(cell[v], (up - um) * inv_dx, o);   // alpha div(u)
-            out[v] = df_from_double(o);
+            out[v] = df_rate(a, o);
         }
-        return finish_cell_rates_df<NF, NDIM, DIR, SIX>(a, idx, out, df_from_double((up - um) * inv_dx), cell, inv_dx, b,
+        return finish_cell_rates_df<NF, NDIM, DIR, SIX>(a, idx, out, df_rate(a, (up - um) * inv_dx), cell, inv_dx, b,
                                                         sd, stg, slot);
     } else {
         Real out[NQ];

@@ -3,6 +3,7 @@
 // index mapping and the FP64 Newton reciprocal.
 #pragma once
 #include <cuda_runtime.h>
+#include <math.h>
 #include <stdint.h>
 #include <string.h>
 
@@ -115,13 +116,23 @@ struct SweepArgs {
     float epsf;
     float inv_dxf[3];
     EosDf ed;               // FP64 kernels: e, eps * 3/4, eps and g.inv_dx in float-float
-    df eps34d, epsd, inv_dxd[3];
+    df eps34d, epsd, inv_dxd[3];    // inv_dxd: times r_scale
+    // FP64 kernels: the accumulator holds rates times r_scale = 2^-r_exp, r_exp the
+    // exponent of the largest 1/dx.  A rate is a flux difference over dx, and scaled so
+    // it is of the size of the flux differences whatever the cell's: unscaled, a flux of
+    // 1e37 overflowed the FP32 range from 1/dx = 34 on
+    int r_exp;
+    float r_scale;
     df kgamd[3], kpinfd[3];     // kgam, kpinf in float-float
 };
 
 // Fill the FP32 and float-float constants of a from its FP64 ones (host, after
-// e, eps, g and the phase constants).
-inline void sweep_set_constants(SweepArgs& a) {
+// e, eps, g and the phase constants).  max_inv_dx: of all cells and directions.
+inline void sweep_set_constants(SweepArgs& a, double max_inv_dx) {
+    a.r_exp = max_inv_dx > 0x1p-100 && max_inv_dx < 0x1p101 ? ilogb(max_inv_dx)
+              : max_inv_dx < 1.0                             ? -100
+                                                             : 100;
+    a.r_scale = ldexpf(1.f, -a.r_exp);
     a.ef.G_N = (float)a.e.G_N;
     a.ef.P_N = (float)a.e.P_N;
     a.ef.A_N = (float)a.e.A_N;
@@ -153,7 +164,7 @@ inline void sweep_set_constants(SweepArgs& a) {
     }
     a.eps34d = df_split(0.75 * a.eps);
     a.epsd = df_split(a.eps);
-    for (int d = 0; d < 3; ++d) a.inv_dxd[d] = df_split(a.g.inv_dx[d]);
+    for (int d = 0; d < 3; ++d) a.inv_dxd[d] = df_split(ldexp(a.g.inv_dx[d], -a.r_exp));
     for (int k = 0; k < 3; ++k) {
         a.kgamd[k] = df_split(a.kgam[k]);
         a.kpinfd[k] = df_split(a.kpinf[k]);

@@ -96,7 +96,7 @@ cudaError_t run(const Geometry& g, const EosConst& e, int ndim, const double* q,
         a.fallback = fallback;
         a.fallback_count = nullptr;
         a.cbc = cbc;
-        sweep_set_constants(a);
+        sweep_set_constants(a, fmax(g.inv_dx[0], fmax(g.inv_dx[1], g.inv_dx[2])));
         a.seg = stream_segment(g.ncell, g.n[d], true);
         a.nseg = (g.n[d] + a.seg - 1) / a.seg;
         rc = launch_sweep<double, NF>(a, ndim, d, s);

@@ -514,6 +514,7 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
                 if constexpr (NONUNIF) {   // this cell's width
                     idx_df = grid_df(GridCol<true>(a.grid[0], a.grid_stride[0], c - 1), kGridInvDx);
                     idx_d = df_to_double(idx_df);
+                    idx_df = df_mul_pow2(idx_df, a.r_scale);
                 }
                 racc.add(finish_cell_df<NF, NDIM, 0, SIX>(a, rowoff + (c - 1), Fm, Fd, dsh_F[NQ][pl], utd, cm1, idx_d,
                                                      idx_df, c - 1, 1));
@@ -897,6 +898,7 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
                 if constexpr (NONUNIF) {   // this cell's width
                     idx_df = grid_df(GridCol<false>(a.grid[DIR], a.grid_stride[DIR], c - 1), kGridInvDx);
                     idx_d = df_to_double(idx_df);
+                    idx_df = df_mul_pow2(idx_df, a.r_scale);
                 }
                 racc.add(finish_cell_df<NF, NDIM, DIR, SIX>(a, basei + (unsigned)(c - 1) * sd, Fm, Fd,
                                                        dsh_F[NQ][eslot(c - 1)][lane], utd, cm1, idx_d, idx_df, c - 1,
