@@ -613,9 +613,7 @@ __device__ __forceinline__ double finish_cell_rates(const SweepArgs& a, long lon
 // A rate formed in FP64 as the accumulator holds it: scaled, float-float; NaN where
 // that is not finite or beyond the FP32 range.
 __device__ __forceinline__ df df_rate(const SweepArgs& a, double r) {
-    r *= df_widen(a.r_scale);
-    const df x = df_from_double_rn(r);
-    return ((unsigned)__double2hiint(r) & 0x7FF00000u) < (1023u + 127u) << 20 ? x : df{NAN, 0.f};
+    return df_from_double_kept(r * df_widen(a.r_scale));
 }
 
 // The rates in out and the face-velocity divergence du come in scaled by
@@ -627,14 +625,14 @@ __device__ __forceinline__ double finish_cell_rates_df(const SweepArgs& a, long 
     using Lay = Layout<NF, NDIM, SIX>;
     constexpr int NS = Lay::NS, NQ = Lay::NQ, IA = Lay::IA;
     if constexpr (SIX) {
-        const df pdu = df_mul(df_from_double(cell[Lay::IE]), du);
+        const df pdu = df_mul(df_from_double_kept(cell[Lay::IE]), du);
         double aN = 1.0;
 #pragma unroll
         for (int k = 0; k < NF - 1; ++k) {
             aN -= cell[IA + k];
-            out[Lay::II + k] = df_add_fast(out[Lay::II + k], df_neg(df_mul(df_from_double(cell[IA + k]), pdu)));
+            out[Lay::II + k] = df_add_fast(out[Lay::II + k], df_neg(df_mul(df_from_double_kept(cell[IA + k]), pdu)));
         }
-        out[Lay::II + NF - 1] = df_add_fast(out[Lay::II + NF - 1], df_neg(df_mul(df_from_double(aN), pdu)));
+        out[Lay::II + NF - 1] = df_add_fast(out[Lay::II + NF - 1], df_neg(df_mul(df_from_double_kept(aN), pdu)));
     }
     if constexpr (NF > 1) {
         if (a.kapila) {
@@ -742,7 +740,7 @@ __device__ __forceinline__ double finish_cell_df(const SweepArgs& a, long long i
     for (int v = 0; v < NQ; ++v) {
         df diff;
         if (v >= IA && v < IA + NF - 1) {
-            const df al = df_from_double_rn(cell[v]);
+            const df al = df_from_double_kept(cell[v]);
             diff = df_add(df_mul(df_add(al, df_neg(Fp[v])), up), df_neg(df_mul(df_add(al, df_neg(Fm[v])), um)));
         } else {
             diff = df_add_fast(Fm[v], df_neg(Fp[v]));
