@@ -320,10 +320,53 @@ __device__ __forceinline__ void stage_finish_operands(const SweepArgs& a, long l
 // doubles), so it is exact and independent of scheduling.  Six-equation model
 // (SIX): the frozen sound speed, r c^2 = A p + B (Sec. 2.3).
 // ---------------------------------------------------------------------------
+// Six-equation model, FP64 form: 1/rho and the internal energy of a cell, and the
+// mixture-law pressure of that energy.  The relaxation needs them too, and since both
+// use these (each operation rounded as written), the primitives a step ends with are
+// those recovered from the state it leaves, bit for bit.
+template <int NF, int NDIM>
+__device__ __forceinline__ void six_energy(const double* q, double& irho, double& eint) {
+    using Lay = Layout<NF, NDIM, true>;
+    double r = q[0], m2 = 0.0;
+#pragma unroll
+    for (int k = 1; k < NF; ++k) r += q[k];
+#pragma unroll
+    for (int d = 0; d < NDIM; ++d) m2 = fma(q[Lay::IM + d], q[Lay::IM + d], m2);
+    irho = rcp_nr(r);
+    eint = fma(-0.5 * m2, irho, q[Lay::IE]);
+}
+template <int NF, int NDIM>
+__device__ __forceinline__ double six_pressure(const double* q, const EosConst& e, double eint) {
+    double G = e.G_N, P = e.P_N;
+#pragma unroll
+    for (int k = 0; k < NF - 1; ++k) {
+        G = fma(q[Layout<NF, NDIM>::IA + k], e.dG[k], G);
+        P = fma(q[Layout<NF, NDIM>::IA + k], e.dP[k], P);
+    }
+    return __dmul_rn(eint - P, rcp_nr(G));
+}
+
 template <int NF, int NDIM, bool SIX = false>
 __device__ __forceinline__ void prims_cell(const double* q, const EosConst& e, double* wv, double& c2) {
     using Lay = Layout<NF, NDIM>;
     constexpr int IM = Lay::IM, IE = Lay::IE, IA = Lay::IA;
+    if constexpr (SIX) {
+        double irho, eint;
+        six_energy<NF, NDIM>(q, irho, eint);
+#pragma unroll
+        for (int v = 0; v < Lay::NS; ++v) wv[v] = q[v];
+#pragma unroll
+        for (int d = 0; d < NDIM; ++d) wv[IM + d] = __dmul_rn(q[IM + d], irho);
+        wv[IE] = six_pressure<NF, NDIM>(q, e, eint);
+        double A = e.A_N, B = e.B_N;
+#pragma unroll
+        for (int k = 0; k < NF - 1; ++k) {
+            A = fma(q[IA + k], e.dA[k], A);
+            B = fma(q[IA + k], e.dB[k], B);
+        }
+        c2 = __dmul_rn(fma(A, wv[IE], B), irho);
+        return;
+    }
     double rho = q[0];
 #pragma unroll
     for (int k = 1; k < NF; ++k) rho += q[k];
@@ -344,17 +387,7 @@ __device__ __forceinline__ void prims_cell(const double* q, const EosConst& e, d
     wv[IE] = p;
 #pragma unroll
     for (int k = 0; k < NF - 1; ++k) wv[IA + k] = q[IA + k];
-    if constexpr (SIX) {
-        double A = e.A_N, B = e.B_N;
-#pragma unroll
-        for (int k = 0; k < NF - 1; ++k) {
-            A = fma(q[IA + k], e.dA[k], A);
-            B = fma(q[IA + k], e.dB[k], B);
-        }
-        c2 = fma(A, p, B) * irho;
-    } else {
-        c2 = fma(G + 1.0, p, P) * iG * irho;
-    }
+    c2 = fma(G + 1.0, p, P) * iG * irho;
 }
 
 // FP32 form: the per-cell FP64 -> FP32 conversions by integer operations

@@ -95,8 +95,8 @@ __global__ void __launch_bounds__(256) prims_kernel(const PrimArgs a) {
 // phases): the start of step 1 and the test E_k0 > a_k0 pinf_k, decided in FP64
 // only where float-float cannot, take none.  STEADY (mixed form) keeps both and
 // the derivatives of step 3 in FP64: there a trace fraction of ~1e-9 feeds FP32
-// arithmetic that tells apart results one FP64 rounding of 1 away.  Returns the pressure of step 4 (of
-// the unchanged state if no phase can relax: the CFL check flags it) and 1/rho.
+// arithmetic that tells apart results one FP64 rounding of 1 away.  If no phase can
+// relax the state is left as it is: the CFL check flags it.
 __device__ __forceinline__ bool energy_above(double E, double x, double pinf, df Ed, df xd, df pinfd) {
     const unsigned big = (1023u + 120u) << 20;   // above 2^120 or not finite: float-float does not hold it
     if (((unsigned)__double2hiint(E) & 0x7FF00000u) < big && ((unsigned)__double2hiint(x) & 0x7FF00000u) < big) {
@@ -107,17 +107,11 @@ __device__ __forceinline__ bool energy_above(double E, double x, double pinf, df
 }
 
 template <int NF, int NDIM, bool STEADY>
-__device__ __forceinline__ void relax6(const RelaxConst& c, const EosConst& e, double* q, double& pressure,
-                                       double& irho) {
+__device__ __forceinline__ void relax6(const RelaxConst& c, const EosConst& e, double* q) {
     using Lay = Layout<NF, NDIM, true>;
-    constexpr int IM = Lay::IM, IE = Lay::IE, IA = Lay::IA, II = Lay::II;
-    double r = q[0], m2 = 0.0;
-#pragma unroll
-    for (int k = 1; k < NF; ++k) r += q[k];
-#pragma unroll
-    for (int d = 0; d < NDIM; ++d) m2 = fma(q[IM + d], q[IM + d], m2);
-    irho = rcp_nr(r);
-    const double eint = fma(-0.5 * m2, irho, q[IE]);
+    constexpr int IA = Lay::IA, II = Lay::II;
+    double irho, eint;
+    six_energy<NF, NDIM>(q, irho, eint);
     double a0[NF];
     df a0d[NF], E0d[NF];
     bool in[NF];
@@ -241,15 +235,11 @@ __device__ __forceinline__ void relax6(const RelaxConst& c, const EosConst& e, d
         }
     }
     // 4. the pressure of the total energy, the phase energies
-    double G = e.G_N, P = e.P_N, an = 1.0;
-#pragma unroll
-    for (int k = 0; k < NF - 1; ++k) {
-        G = fma(q[IA + k], e.dG[k], G);
-        P = fma(q[IA + k], e.dP[k], P);
-        an -= q[IA + k];
-    }
-    pressure = (eint - P) * rcp_nr(G);
     if (any) {
+        const double pressure = six_pressure<NF, NDIM>(q, e, eint);
+        double an = 1.0;
+#pragma unroll
+        for (int k = 0; k < NF - 1; ++k) an -= q[IA + k];
 #pragma unroll
         for (int k = 0; k < NF; ++k) q[II + k] = (k < NF - 1 ? q[IA + k] : an) * fma(c.G[k], pressure, c.P[k]);
     }
@@ -263,7 +253,7 @@ __device__ __forceinline__ void relax6(const RelaxConst& c, const EosConst& e, d
 template <typename Real, int NF, int NDIM, bool RATE>
 __global__ void __launch_bounds__(256) relax_prims_kernel(const PrimArgs a, const RelaxConst c) {
     using Lay = Layout<NF, NDIM, true>;
-    constexpr int NS = Lay::NS, NQ = Lay::NQ, IM = Lay::IM, IE = Lay::IE, IA = Lay::IA, II = Lay::II;
+    constexpr int NS = Lay::NS, NQ = Lay::NQ, IA = Lay::IA, II = Lay::II;
     pdl_wait();
     const long long nc = a.g.ncell;
     double rate = 0.0;
@@ -272,33 +262,16 @@ __global__ void __launch_bounds__(256) relax_prims_kernel(const PrimArgs a, cons
     Real* w = static_cast<Real*>(a.w);
     for (long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x; i < nc;
          i += (long long)gridDim.x * blockDim.x) {
-        double q[NQ], p, irho;
+        double q[NQ];
 #pragma unroll
         for (int v = 0; v < NQ; ++v) q[v] = qs[v * nc + i];
-        relax6<NF, NDIM, sizeof(Real) == 4>(c, a.e, q, p, irho);
+        relax6<NF, NDIM, sizeof(Real) == 4>(c, a.e, q);
 #pragma unroll
         for (int v = IA; v < IA + NF - 1; ++v) qs[v * nc + i] = q[v];
 #pragma unroll
         for (int v = II; v < II + NF; ++v) qs[v * nc + i] = q[v];
-        Real wv[NS], c2 = 0;
-        if constexpr (sizeof(Real) == 8) {
-#pragma unroll
-            for (int v = 0; v < NS; ++v) wv[v] = q[v];
-#pragma unroll
-            for (int d = 0; d < NDIM; ++d) wv[IM + d] = q[IM + d] * irho;
-            wv[IE] = p;
-            if (RATE) {
-                double A = a.e.A_N, B = a.e.B_N;
-#pragma unroll
-                for (int k = 0; k < NF - 1; ++k) {
-                    A = fma(q[IA + k], a.e.dA[k], A);
-                    B = fma(q[IA + k], a.e.dB[k], B);
-                }
-                c2 = fma(A, p, B) * irho;
-            }
-        } else {
-            prims_cell<NF, NDIM, true>(q, a.e, wv, c2);
-        }
+        Real wv[NS], c2;
+        prims_cell<NF, NDIM, true>(q, a.e, wv, c2);   // shares 1/rho, energy and pressure with the relaxation
 #pragma unroll
         for (int v = 0; v < NS; ++v) w[v * nc + i] = wv[v];
         if (RATE) {
