@@ -182,9 +182,9 @@ __device__ __forceinline__ void dfs_edges(const SweepArgs& a, int dir, int c, in
         const GridCol<VALUE_MAJOR> grow(a.grid[dir], a.grid_stride[dir], c);
         I = weno5_increments_nu_pair(D, a.epsd, grow);
     } else if constexpr (ORDER == 5) {
-        I = weno5_increments_pair(D, a.eps34d);
+        I = weno5_increments_pair<SIX>(D, a.eps34d);
     } else {
-        I = weno3_increments_pair(D[1], D[2], a.epsd);
+        I = weno3_increments_pair<SIX>(D[1], D[2], a.epsd);
     }
     if (SIX && q >= Layout<NF, NDIM>::IA && q < Layout<NF, NDIM>::IA + NF - 1) {
         eL = df_pack(vc + df_to_double(df2_x(I)));

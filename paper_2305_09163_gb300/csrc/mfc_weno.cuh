@@ -46,6 +46,14 @@ namespace mfc {
 // -> 2.91 / 2.78 ms, error unchanged).
 // The indicators are formed as b0 = D0^2 + D1 (5/2 D1 - 11/4 D0), b2 mirrored, and
 // b1 = D1^2 + D2 (D2 - 5/4 D1): two products instead of three.
+//
+// EVEN: m is the whole float-float minimum instead of its hi part, so the largest
+// weights are exactly one and, where the stencil is smooth against eps, the increment
+// is the exact one.  For edges that are then rounded to FP64 beside the cell value
+// (six-equation volume fractions): next to a trace phase the differences are a few
+// units in the last place of 1, increments of half a unit are common, and each
+// one rounded the wrong way shows in the trace phase's energy.
+template <bool EVEN = false>
 __device__ __forceinline__ df2 weno5_increments_pair(const df (&D)[4], df e) {
     const df2 X0 = df2_make(D[0], df_neg(D[3])), X1 = df2_make(D[1], df_neg(D[2]));
     const df2 X2 = df2_swap(df2_neg(X1)), X3 = df2_swap(df2_neg(X0));   // (D2, -D1), (D3, -D0)
@@ -54,9 +62,19 @@ __device__ __forceinline__ df2 weno5_increments_pair(const df (&D)[4], df e) {
     const df b1 = df_sum(df_square(D[1]), df_prod(D[2], df_sum(D[2], df_scale(D[1], -1.25f))));
     const df2 T = df2_sum(B, df2_make(e, e));                            // (t0, t2)
     const df t1 = df_sum(b1, e);
-    const float m = fminf(T.hi.x, fminf(t1.hi, T.hi.y));
-    const df2 Q = df2_norm(df2_square(df2_quot_f(f2(m), T)));            // (q0, q2)
-    const df q1 = df_norm(df_scale(df_square(df_quot_f(m, t1)), 6.f));
+    df2 G;
+    df g1;
+    if constexpr (EVEN) {
+        const df t02 = T.hi.y < T.hi.x ? df2_y(T) : df2_x(T), m = t1.hi < t02.hi ? t1 : t02;
+        G = df2_quot(df2_make(m, m), T);
+        g1 = df_quot(m, t1);
+    } else {
+        const float m = fminf(T.hi.x, fminf(t1.hi, T.hi.y));
+        G = df2_quot_f(f2(m), T);
+        g1 = df_quot_f(m, t1);
+    }
+    const df2 Q = df2_norm(df2_square(G));                               // (q0, q2)
+    const df q1 = df_norm(df_scale(df_square(g1), 6.f));
     const df2 Q1 = df2_make(q1, q1);
     const df2 W2 = df2_scale(df2_swap(Q), f2(3.f));                      // (3 q2, 3 q0)
     const df2 P0 = df2_sum(df2_scale(X1, f2(5.f)), df2_mul_pow2(X0, f2(-2.f)));
@@ -141,11 +159,18 @@ __device__ __forceinline__ void weno5_edges(float vc, const float D[4], float ep
 // ---------------------------------------------------------------------------
 // The two WENO3 increments (c+1/2 in lane x, c-1/2 in lane y): lane y evaluates
 // the c+1/2 formula on the mirrored differences (-b, -a).
+template <bool EVEN = false>
 __device__ __forceinline__ df2 weno3_increments_pair(df A, df Bd, df E) {
     const df2 X = df2_make(A, df_neg(Bd)), Y = df2_make(Bd, df_neg(A));
     const df2 T = df2_sum(df2_square(df2_make(A, Bd)), df2_make(E, E));   // (t0, t1)
-    const float m = fminf(T.hi.x, T.hi.y);
-    const df2 S = df2_norm(df2_square(df2_quot_f(f2(m), T)));        // (s0, s1)
+    df2 G;
+    if constexpr (EVEN) {
+        const df m = T.hi.y < T.hi.x ? df2_y(T) : df2_x(T);
+        G = df2_quot(df2_make(m, m), T);
+    } else {
+        G = df2_quot_f(f2(fminf(T.hi.x, T.hi.y)), T);
+    }
+    const df2 S = df2_norm(df2_square(G));                           // (s0, s1)
     const df2 S2 = df2_mul_pow2(df2_swap(S), f2(2.f));               // (2 s1, 2 s0)
     const df2 num = df2_sum(df2_prod(S, X), df2_prod(S2, Y));
     const df2 den = df2_mul_pow2(df2_sum(S, S2), f2(2.f));
