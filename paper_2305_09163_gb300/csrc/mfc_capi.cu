@@ -117,6 +117,7 @@ size_t real_size(const mfc_ctx* c) { return is_f32(c) ? sizeof(float) : sizeof(d
 bool nonuniform(const mfc_ctx* c) { return c->grid[0] || c->grid[1] || c->grid[2]; }
 
 int auto_segment(const mfc_ctx* c, int dir) {
+    if (dir == 0) return c->n[0];   // the x sweep has its own split
     if (c->seg_override > 0) return c->seg_override;
     const bool stream = c->six || nonuniform(c) || c->yz_stream != 0;   // the rule of launch_sweep
     return stream ? stream_segment(c->ncell, c->n[dir], !is_f32(c)) : marching_segment(c->ncell, c->n[dir]);

@@ -97,7 +97,7 @@ cudaError_t run(const Geometry& g, const EosConst& e, int ndim, const double* q,
         a.fallback_count = nullptr;
         a.cbc = cbc;
         sweep_set_constants(a, fmax(g.inv_dx[0], fmax(g.inv_dx[1], g.inv_dx[2])));
-        a.seg = stream_segment(g.ncell, g.n[d], true);
+        a.seg = d == 0 ? g.n[0] : stream_segment(g.ncell, g.n[d], true);   // the x sweep has its own split
         a.nseg = (g.n[d] + a.seg - 1) / a.seg;
         rc = launch_sweep<double, NF>(a, ndim, d, s);
         if (rc != cudaSuccess) return rc;
