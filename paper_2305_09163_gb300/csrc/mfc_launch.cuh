@@ -46,7 +46,9 @@ cudaError_t launch_pdl(void (*kernel)(P...), unsigned blocks, int threads, size_
     at.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
+    const cudaError_t rc = cudaLaunchKernelEx(&cfg, kernel, args...);
+    if (rc != cudaSuccess) cudaGetLastError();   // reported here, not once more to whoever asks next
+    return rc;
 }
 
 inline size_t stage_bytes_rt(int mask, int nq, size_t real_size) {
