@@ -89,7 +89,8 @@ typedef enum { MFC_FP64 = 0, MFC_MIXED = 1, MFC_LEARNED = 2 } mfc_precision;
 /* Create a context (Sec. 3.1: uniform structured grid; Sec. 3.3: ghost-cell
  * boundaries; Sec. 2.1: stiffened-gas fluids).
  *   nx, ny, nz   cells per direction; 1D: ny = nz = 1, 2D: nz = 1.  Every
- *                active direction needs at least 3 cells.
+ *                active direction needs at least 3 cells; fewer than 2^32
+ *                in all.
  *   lo, hi       domain corners [3] (only active directions are used).
  *   bc           [6] boundary types for -x,+x,-y,+y,-z,+z (mfc_bc); periodic
  *                must be set on both faces of a direction.  Characteristic

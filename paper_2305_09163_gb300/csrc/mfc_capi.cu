@@ -493,7 +493,7 @@ mfc_status mfc_init(mfc_ctx** out, int nx, int ny, int nz, const double lo[3], c
         if (!(gamma[k] > 1.0) || !(pi_inf[k] >= 0.0) || !std::isfinite(gamma[k]) || !std::isfinite(pi_inf[k]))
             return MFC_ERR_ARG;
     const long long ncell = (long long)nx * ny * nz;
-    if (ncell > (1LL << 34)) return MFC_ERR_ARG;
+    if ((long long)nx * ny > kMaxStateCells || ncell > kMaxStateCells) return MFC_ERR_ARG;
 
     mfc_ctx* c = new mfc_ctx();
     for (int d = 0; d < 3; ++d) {

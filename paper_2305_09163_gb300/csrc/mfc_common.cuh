@@ -21,6 +21,9 @@ struct Geometry {
     double inv_dx[3];
 };
 
+// The most cells of a state: the y/z sweeps index them with 32 bits.
+constexpr long long kMaxStateCells = (1LL << 32) - 1;
+
 // Mixture closure written as Gamma = G_N + sum_{k<N} alpha_k dG_k, with
 // G_k = 1/(gamma_k - 1) and P_k = gamma_k pinf_k/(gamma_k - 1); this is
 // sum_k alpha_k G_k with alpha_N = 1 - sum_{k<N} alpha_k (Sec. 2.1).

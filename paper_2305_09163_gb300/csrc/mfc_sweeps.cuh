@@ -645,8 +645,7 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
     // lanes run over the flat transverse plane (x fastest), so only the plane's
     // last warp has idle lanes, whatever the row length
     const int nd = a.g.n[DIR];
-    // 32-bit indices (registers): 2D and 3D states take at least 112 bytes per
-    // cell, so the device's memory holds fewer than 2^32 cells and, of three
+    // 32-bit indices (registers): a state has at most kMaxStateCells cells and, of three
     // planes or rows at least, fewer than 2^31 in one
     const int plane = (int)(a.g.ncell / nd);
     const int ncol = (plane + 31) >> 5;

@@ -60,3 +60,12 @@ def test_invalid_init_arguments_are_rejected_without_a_gpu():
         with pytest.raises(m.MFCError) as ei:
             m.mfc_init(kw["n"], kw["lo"], kw["hi"], kw["bc"], kw["gamma"], kw["pi_inf"], kw["precision"], None)
         assert ei.value.status == m.MFC_ERR_ARG
+
+
+@pytest.mark.parametrize("n", [(1625, 1625, 1627), (65536, 65536, 1), (3, 65536, 65536), (3000000, 3000000, 3000000)])
+def test_more_cells_than_the_kernels_index_are_rejected(n):
+    """2^32 cells and more: refused as a size, before any allocation is tried."""
+    import paper_2305_09163_gb300 as m
+    with pytest.raises(m.MFCError) as ei:
+        m.mfc_init(n, (0, 0, 0), (1, 1, 1), (1,) * 6, (1.4,), (0.0,), 0, None)
+    assert ei.value.status == m.MFC_ERR_ARG
