@@ -644,14 +644,17 @@ __global__ void __launch_bounds__(128) harvest_kernel(const double* __restrict__
 }
 
 // n / d from the FP64 Newton reciprocal r of d, finished with the exact residual
-// (Markstein): the rounding of a division; anything not finite is divided (out of
-// line: inlined, the division ran speculatively in every lane, 58 FP64
-// instructions per cell instead of 27).
+// (Markstein): the rounding of a division while the residual is representable (|n| from
+// 2^-900 on) and the quotient normal.  A zero n is its own sign's quotient; the rest is
+// divided (out of line: inlined, the division ran speculatively in every lane, 58
+// FP64 instructions per cell instead of 27).
 __device__ __noinline__ double div_slow(double n, double d) { return n / d; }
 __device__ __forceinline__ double div_by(double n, double d, double r) {
     const double q = n * r;
     const double res = fma(fma(-q, d, n), r, q);
-    return abs_hi(res) < 0x7FF00000u ? res : div_slow(n, d);
+    if (abs_hi(n) >= 0x07B00000u && abs_hi(res) - 0x00100000u < 0x7FE00000u) return res;
+    if (((__double_as_longlong(n) | __double_as_longlong(q)) << 1) == 0) return q;
+    return div_slow(n, d);
 }
 
 // FP64 primitive recovery for output; the six-equation model (SIX) appends the
