@@ -443,9 +443,10 @@ __device__ __forceinline__ df2 weno5_right_pair(df2 X0, df2 X1, df2 X2, df2 X3, 
 }
 
 // One sample's outputs in plain FP64, for values outside the range of the
-// float-float form below: differences of 1e18 and more or of less than 2^-60 of
-// them all, non-finite values, eps outside [1e-30, 1].  f6: per fine face the six
-// values across it.
+// float-float form below: a centre value or difference of 2^59 (5.8e17) and more or
+// not finite, a stencil that spans less than 2^-45 (2.8e-14; the sensor's 1e-6 s^2 would
+// fall among the FP32 subnormals, with 9 bits left at 2^-60), eps outside [1e-30, 1],
+// tau outside [1e-30, 1e30].  f6: per fine face the six values across it.
 __device__ __noinline__ void harvest_sample_f64(const double* st, const double* f6, int ntr, double eps, double tau,
                                                 float* x, float* ph, float* to, float* so, float* jo) {
     double tgt = 0.0;
@@ -585,7 +586,7 @@ __global__ void __launch_bounds__(128) harvest_kernel(const double* __restrict__
             big = max(big, abs_hi(e[t][j]));
         }
     big = max(big, (unsigned)(sb >> 32));
-    constexpr unsigned kMax = (1023u + 59u) << 20, kMin = (1023u - 60u) << 20;   // 5.8e17, 8.7e-19
+    constexpr unsigned kMax = (1023u + 59u) << 20, kMin = (1023u - 45u) << 20;   // 5.8e17, 2.8e-14
     const bool flat = !(s > 1e-7 * fabs(c)) || !(s > 1e-300);
     if (!eps_in_range || big >= kMax || (!flat && (unsigned)(sb >> 32) < kMin)) {
         harvest_sample_f64(st, &f6[0][0], NTR, eps, tau, x, ph, &tv, &sv, &jv);
