@@ -653,6 +653,32 @@ def _form_entry(r, ws, cells, neq, head_ms=None):
     return e
 
 
+def summary(line):
+    """The result line: the headline with its configuration, end-to-end figure and
+    clocks, and every other form and configuration as [ms per step, grind time].  The
+    whole record (rooflines, per-kernel times, notes) is 20 KB, more than what reads
+    the end of a run's output keeps, and goes to stderr."""
+    def short(v):
+        if isinstance(v, float):
+            return float("%.6g" % v)
+        if isinstance(v, dict):
+            return {k: short(x) for k, x in v.items()}
+        return [short(x) for x in v] if isinstance(v, list) else v
+
+    out = {k: line[k] for k in ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+                                "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config",
+                                "cell_updates_per_s", "gpu_launches", "kernels_ms", "clocks")}
+    if line["roofline"]:
+        out["roofline"] = {k: line["roofline"][k] for k in ("bound", "resource", "achieved", "peak", "unit", "frac",
+                                                            "flop_tflops", "traffic", "ncu")}
+    for k in ("e2e", "cpu_baseline"):
+        if k in line:
+            out[k] = {f: v for f, v in line[k].items() if not isinstance(v, dict)}
+    for k in ("forms", "configs"):
+        out[k] = {f: [r["ms_per_step"], r["grind"]] for f, r in line[k].items()}
+    return short(out)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -816,7 +842,8 @@ def main():
     if rank == 0 and ws == 1 and not args.no_cpu_baseline:
         line["cpu_baseline"] = cpu_baseline_sample(wl, w_host)
     if rank == 0:
-        print(json.dumps(line))
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(summary(line)))
     if ws > 1:
         import torch.distributed as dist
         dist.destroy_process_group()
