@@ -235,8 +235,8 @@ __device__ __forceinline__ void relax6(const RelaxConst& c, const EosConst& e, d
         }
     }
     // 4. the pressure of the total energy, the phase energies
+    const double pressure = six_pressure<NF, NDIM>(q, e, eint);   // outside the test: the recovery takes it over
     if (any) {
-        const double pressure = six_pressure<NF, NDIM>(q, e, eint);
         double an = 1.0;
 #pragma unroll
         for (int k = 0; k < NF - 1; ++k) an -= q[IA + k];
