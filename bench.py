@@ -86,22 +86,22 @@ SCHEDULERS = 152 * 4
 # Warp instructions per cell of the FP64 WENO5 sweeps (x, y, z; 3D, two
 # fluids, smsp__inst_executed.sum / cells of one ncu capture).  Re-measured
 # whenever the FP64 sweeps change: NCU_FP64_SWEEPS says which capture.
-FP64_SWEEP_WARP_INST_PER_CELL = (130.5, 130.4, 146.7)
+FP64_SWEEP_WARP_INST_PER_CELL = (130.6, 133.3, 151.5)
 # From the same capture: FP64-pipe and FP32 (fma) pipe activity of the sweeps
 # (mean over x, y, z) and DRAM bytes per cell per launch (the z sweep of an RK
 # stage also writes the next stage's primitives).
-FP64_SWEEP_PIPE_FP64 = 0.279
-FP64_SWEEP_PIPE_FMA = 0.642
-FP64_SWEEP_DRAM_BYTES_PER_CELL = (101.7 + 156.8 + 331.1) / 3.0
+FP64_SWEEP_PIPE_FP64 = 0.276
+FP64_SWEEP_PIPE_FMA = 0.646
+FP64_SWEEP_DRAM_BYTES_PER_CELL = (101.8 + 156.7 + 331.2) / 3.0
 NCU_FP64_SWEEPS = "profiles/sweep_fp64_shock_bubble_160.md"
 # The same count for the other FP64 forms (x, y, z; 160^3 shock-bubble, RK
 # stage 2; profiles/sweep_fp64_forms_shock_bubble_160.md).
 FP64_SWEEP_WARP_INST_PER_CELL_FORM = {
-    "fp64_weno3": (86.5, 90.3, 106.6),
-    "fp64_kapila": (142.5, 141.8, 158.0),
-    "fp64_stretched": (169.1, 160.8, 177.5),
-    "fp64_cbc": (132.3, 130.9, 147.1),
-    "fp64_six": (145.6, 149.1, 161.6),
+    "fp64_weno3": (86.6, 91.8, 109.9),
+    "fp64_kapila": (142.6, 144.6, 162.8),
+    "fp64_stretched": (168.6, 162.7, 181.2),
+    "fp64_cbc": (133.0, 133.8, 151.9),
+    "fp64_six": (147.7, 151.2, 166.1),
 }
 NCU_FP64_FORMS = "profiles/sweep_fp64_forms_shock_bubble_160.md"
 # Nominal FP32 peak: 152 SMs x 128 FMA/clk x 2 FLOP x 2.07 GHz

@@ -13,12 +13,13 @@ constexpr int kElemThreads = 256;
 // kernel walks.  A CTA starts two slots early (both faces of its first cell), so
 // k chunks finish 128 k - 2 slots; owning exactly that many leaves no nearly
 // empty last chunk (2,048 owned slots took 17 chunks for the work of 16.02).
-// Long runs save those two slots, short ones fill the chip: a chunk takes ~10 us
-// alone on an SM and ~4.3 us with four CTAs sharing it, and with the fixed 16
-// chunks a 1000-cell row ran on one SM (79 us per launch) and a 65,000-cell block
-// on half of them.  So k grows only once every SM has 16 CTAs to run, four
-// times what it holds, where the walk's end is a small part; past 16 the two
-// slots are 0.1% and nothing is left to save.
+// Long runs save those two slots, short ones fill the chip: a launch of one
+// chunk per CTA takes 10.7 us (1000 cells), a lone CTA's long walk ~6 us a chunk and
+// four CTAs sharing an SM ~4.3 us for each, and with the fixed 16 chunks a 1000-cell row ran on one SM (79 us per launch) and a
+// 65,000-cell block on half of them.  So k grows only once every SM has 16 CTAs to
+// run, three to four times what it holds (five of the uniform two-fluid FP64 form, four
+// of the others), where the walk's end is a small part; past 16 the two slots are 0.1%
+// and nothing is left to save.
 constexpr long long kStreamMaxChunks = 16;
 constexpr long long kStreamMinBlocks = 152LL * 16;
 

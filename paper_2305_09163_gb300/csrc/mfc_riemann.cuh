@@ -227,8 +227,8 @@ struct MixDf {
 };
 
 // Fluxes and face velocity in float-float; the volume-fraction rows of F hold the
-// upwind fraction itself (their flux is that times ut; finish_cell_rates_df takes
-// them so).  Returns whether the flux took the left state (useL).  A product that enters a sum is normalised, one that only
+// upwind fraction itself (their flux is that times ut; finish_cell_df takes them
+// so).  Returns whether the flux took the left state (useL).  A product that enters a sum is normalised, one that only
 // meets further products or is a flux is not (mfc_df.cuh): with unnormalised terms
 // in the sums the right-hand side's error against 64 bits grew by 25% (the kinetic
 // energy's do not show).

@@ -621,8 +621,8 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
     // z 3449 -> 3042 us; 100x90x77: y 124.0 -> 122.5, z 140.9 -> 138.5.  Where one
     // wave of blocks holds the whole grid the chain of each chunk counts instead of
     // the FP64 pipe: 48x41x33 y 26.1 -> 24.5, z 26.8 -> 29.8.  Not the six-equation
-    // model (its interior edge values are FP64 sums) nor the x sweep, whose rows stay
-    // in value-major FP64 for its staged loads
+    // model (its volume-fraction edges are FP64 sums) nor the x sweep, which has no ring:
+    // it would split each value five times, once for every stencil that reads it
     constexpr bool TRI = sizeof(Real) == 8 && !LEARNED && !SIX;
     __shared__ Real ring[RING][NS][32];
     __shared__ float ring_lo[TRI ? RING : 1][TRI ? NS : 1][32];
