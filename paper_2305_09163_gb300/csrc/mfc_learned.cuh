@@ -148,7 +148,7 @@ __device__ __forceinline__ int learned_cell_edges(const Stencil& stencil, float 
 template <int NF, int NDIM, int DIR, typename LoadJ>
 __device__ __forceinline__ void face_flux_learned(const SweepArgs& a, const EosR<float>& e, const float* Ll,
                                                   const float* Rl, const LoadJ& loadJ, const float* cl,
-                                                  const float* cr, float* F, float& ut) {
+                                                  const float* cr, float* F, float& ut, bool count) {
     constexpr int NS = Layout<NF, NDIM>::NS;
     float fl[NS], fr[NS];
 #pragma unroll
@@ -171,7 +171,7 @@ __device__ __forceinline__ void face_flux_learned(const SweepArgs& a, const EosR
                 }
                 mL = mixture<float, NF, NDIM>(fl, e);
                 mR = mixture<float, NF, NDIM>(fr, e);
-                count_fallback(a.fallback_count);
+                if (count) count_fallback(a.fallback_count);
             }
         }
     }

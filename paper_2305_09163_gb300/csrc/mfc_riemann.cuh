@@ -381,10 +381,12 @@ __device__ __forceinline__ void count_fallback(unsigned long long* counter) {
 }
 
 // Face flux between reconstructed states (with the optional first-order
-// fallback to the two cell values cl | cr).
+// fallback to the two cell values cl | cr).  count: this lane counts the face if it
+// falls back (false where a neighbouring CTA or segment computes it too and counts
+// it, and on lanes past the plane's end).
 template <typename Real, int NF, int NDIM, int DIR, bool SIX = false>
 __device__ __forceinline__ void face_flux(const SweepArgs& a, const EosR<Real>& e, const Real* eLs, const Real* eRs,
-                                          const Real* cl, const Real* cr, Real* F, Real& ut) {
+                                          const Real* cl, const Real* cr, Real* F, Real& ut, bool count) {
     constexpr int NS = Layout<NF, NDIM>::NS;
     Mix<Real> mL = mixture<Real, NF, NDIM, SIX>(eLs, e);
     Mix<Real> mR = mixture<Real, NF, NDIM, SIX>(eRs, e);
@@ -395,7 +397,7 @@ __device__ __forceinline__ void face_flux(const SweepArgs& a, const EosR<Real>& 
     if constexpr (sizeof(Real) == 4) {
         // FP32: a per-lane branch (the compiler schedules this form best)
         if (first) {
-            count_fallback(a.fallback_count);
+            if (count) count_fallback(a.fallback_count);
             Real fl[NS], fr[NS];
 #pragma unroll
             for (int v = 0; v < NS; ++v) { fl[v] = cl[v]; fr[v] = cr[v]; }
@@ -417,7 +419,7 @@ __device__ __forceinline__ void face_flux(const SweepArgs& a, const EosR<Real>& 
             sr[v] = first ? cr[v] : eRs[v];
         }
         if (first) {
-            count_fallback(a.fallback_count);
+            if (count) count_fallback(a.fallback_count);
             mL = mixture<Real, NF, NDIM, SIX>(sl, e);
             mR = mixture<Real, NF, NDIM, SIX>(sr, e);
         }
@@ -440,7 +442,7 @@ __device__ __forceinline__ void face_flux(const SweepArgs& a, const EosR<Real>& 
 // only where a face falls back, so the two cells' states need not be at hand.
 template <int NF, int NDIM, int DIR, bool SIX = false, typename Cells>
 __device__ __forceinline__ void face_flux_df(const SweepArgs& a, const df* eLs, const df* eRs, const Cells& cells,
-                                             df* F, df& ut) {
+                                             df* F, df& ut, bool count) {
     using Lay = Layout<NF, NDIM>;
     constexpr int NS = Lay::NS;
     const EosDf& e = a.ed;
@@ -464,7 +466,7 @@ __device__ __forceinline__ void face_flux_df(const SweepArgs& a, const df* eLs, 
     MixDf mR = mixture_df<NF, NDIM, SIX>(sr, e);
     const bool first = a.fallback && !(face_state_ok_df<NF, NDIM>(sl, mL) && face_state_ok_df<NF, NDIM>(sr, mR));
     if (first) {
-        count_fallback(a.fallback_count);
+        if (count) count_fallback(a.fallback_count);
 #pragma unroll
         for (int v = 0; v < NS; ++v) {
             const double cl = cells(v, 0), cr = cells(v, 1);

@@ -111,9 +111,9 @@ __global__ void __launch_bounds__(128) sweep_kernel(const SweepArgs a) {
                             Rj[v] = eRJ[v];
                         }
                     },
-                    cm1, vc, F, ut);
+                    cm1, vc, F, ut, active && (c < s1 || s1 == nd));
             else
-                face_flux<Real, NF, NDIM, DIR>(a, e, eLprev, eR, cm1, vc, F, ut);
+                face_flux<Real, NF, NDIM, DIR>(a, e, eLprev, eR, cm1, vc, F, ut, c < s1 || s1 == nd);
             if (c >= s0 + 1 && active)
                 racc.add(finish_cell<Real, NF, NDIM, DIR>(a, base + (long long)(c - 1) * sd, Fprev, F, utprev, ut, cm1,
                                                           inv_dx, c - 1, sd));
@@ -472,7 +472,7 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
                 const double x = __ldg(w + v * nc + rowoff + m);
                 return v == IM && flip ? -x : x;
             };
-            face_flux_df<NF, NDIM, 0, SIX>(a, lftd, erd, cells, Fd, utd);
+            face_flux_df<NF, NDIM, 0, SIX>(a, lftd, erd, cells, Fd, utd, s >= own0);
 #pragma unroll
             for (int q = 0; q < NQ; ++q) dsh_F[q][pos] = Fd[q];
             dsh_F[NQ][pos] = utd;
@@ -495,9 +495,9 @@ __device__ __forceinline__ void sweep_x_stream_body(const SweepArgs& a) {
                             Rj[q] = sh_eRJ[q][t];
                         }
                     },
-                    cm1, cell, F, ut);
+                    cm1, cell, F, ut, s >= own0);
             } else {
-                face_flux<Real, NF, NDIM, 0, SIX>(a, e, lft, eR, cm1, cell, F, ut);
+                face_flux<Real, NF, NDIM, 0, SIX>(a, e, lft, eR, cm1, cell, F, ut, s >= own0);
             }
 #pragma unroll
             for (int q = 0; q < NQ; ++q) sh_F[q][pos] = F[q];
@@ -848,7 +848,7 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
                 const double x = __ldg(w + v * nc + basei + (unsigned)m * sd);
                 return v == IM + DIR && flip ? -x : x;
             };
-            face_flux_df<NF, NDIM, DIR, SIX>(a, lftd, erd, cells, Fd, utd);
+            face_flux_df<NF, NDIM, DIR, SIX>(a, lftd, erd, cells, Fd, utd, active && (c < s1 || s1 == nd));
 #pragma unroll
             for (int q = 0; q < NQ; ++q) dsh_F[q][eslot(c)][lane] = Fd[q];
             dsh_F[NQ][eslot(c)][lane] = utd;
@@ -871,9 +871,9 @@ __device__ __forceinline__ void sweep_yz_stream_body(const SweepArgs& a) {
                             Rj[q] = sh_eRJ[q][row][lane];
                         }
                     },
-                    cm1, cell, F, ut);
+                    cm1, cell, F, ut, active && (c < s1 || s1 == nd));
             } else {
-                face_flux<Real, NF, NDIM, DIR, SIX>(a, e, lft, eR, cm1, cell, F, ut);
+                face_flux<Real, NF, NDIM, DIR, SIX>(a, e, lft, eR, cm1, cell, F, ut, active && (c < s1 || s1 == nd));
             }
 #pragma unroll
             for (int q = 0; q < NQ; ++q) sh_F[q][eslot(c)][lane] = F[q];
