@@ -228,10 +228,13 @@ __device__ __forceinline__ void relax6(const RelaxConst& c, const EosConst& e, d
                 f64 += ak[k];
                 fp += dak[k];
             }
+            // f' ~ 1/p leaves FP32 only for pressures beyond 1e30 (a phase energy that does
+            // not belong to the cell's total energy): the fractions at p0 stand then
+            const bool in_range = fabsf(fp) >= 0x1p-100f && fabsf(fp) <= 0x1p100f;
             const float dp = -narrow_rn(f64) * rcp_approx(fp);
 #pragma unroll
             for (int k = 0; k < NF - 1; ++k)
-                if (in[k]) q[IA + k] = ak[k] + df_widen(dak[k] * dp);
+                if (in[k]) q[IA + k] = ak[k] + df_widen(in_range ? dak[k] * dp : 0.f);
         }
     }
     // 4. the pressure of the total energy, the phase energies
